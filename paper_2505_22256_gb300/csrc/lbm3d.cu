@@ -623,39 +623,87 @@ __global__ void k3_set(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags, cons
     }
 }
 
-// f = f^eq(rho_k, 0) written straight into the post-collision buffer as the pull expects it (the
-// state k3_feq + k3_set give, bit for bit, without the [38][N] transfer scratch): the stored f*_i
-// at x is w_i rho(x + e_i), or w_i rho(x) when x + e_i is solid (the link comes back by
-// bounce-back), and 0 at solid nodes.
-template <class S, class R>
-__global__ void k3_set_rest(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags, const double* __restrict__ rA,
-                            const double* __restrict__ rB, Pair<S>* __restrict__ fs) {
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
-    const long long s = ((long long)z * g.ny + y) * g.nx + x;
-    const uint32_t fl = flags[s];
-    for (int i = 0; i < 19; ++i) {
-        V2<R> v{(R)0, (R)0};
-        if (!(fl & k3Solid)) {
-            const bool bl = i > 0 && ((fl >> (opp3(i) - 1)) & 1u);
-            const long long t = (bl || i == 0) ? s : site(g, x + e3x(i), y + e3y(i), z + e3z(i));
-            v = V2<R>{(R)(w19(i) * rA[t]), (R)(w19(i) * rB[t])};
-        }
-        if (fl & k3Solid) store_pair<S, R>(fs + (long long)i * g.N + s, (R)0, (R)0);
-        else st3<S, R>(fs + (long long)i * g.N + s, v, P, i);
-    }
-}
+// f = f^eq(rho_k, 0) written straight into the post-collision buffer as the pull expects it: the
+// stored f*_i at x is w_i rho(x + e_i), or w_i rho(x) when x + e_i is solid (the link comes back by
+// bounce-back), minus the storage shift, and 0 at solid nodes.  The value is (R)(w_i rho) with an FP64
+// product.  1/18 and 1/36 in FP64 are a factor of two apart, so the axis populations are exactly twice
+// q = (R)(rho / 36): per node and component one FP64 product and conversion for q and one for the rest
+// population, instead of 19 (the pass ran at the FP64 pipe's rate, two operations per SM and cycle:
+// 1.61 ms on 200 x 200 x 280 in FP32, where its 168 B per node take 0.28 ms of HBM time; now 0.36 ms).
+// A q so small that scaling it up could differ from rounding the larger product takes the direct form.
+//
+// A block of 32 x 8 columns marches along kR3Z planes of z; q of the plane ahead, with a halo of one
+// node, goes into a ring of four shared-memory planes, one barrier per plane.
+constexpr int kR3X = 32, kR3Y = 8, kR3T = kR3X * kR3Y, kR3Z = 16;
+constexpr int kR3HX = kR3X + 2, kR3P = kR3HX * (kR3Y + 2), kR3N = (kR3P + kR3T - 1) / kR3T;
 
-template <class R>
-__global__ void k3_feq(Geo3 g, const uint8_t* __restrict__ solid, const double* __restrict__ rA, const double* __restrict__ rB,
-                       double* __restrict__ f) {
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
-    const long long s = ((long long)z * g.ny + y) * g.nx + x;
-    const bool sol = solid[s] != 0;
-    for (int i = 0; i < 19; ++i) {
-        f[(long long)i * g.N + s] = sol ? 0.0 : w19(i) * rA[s];
-        f[(long long)(19 + i) * g.N + s] = sol ? 0.0 : w19(i) * rB[s];
+template <class S, class R>
+__global__ void __launch_bounds__(kR3T) k3_set_rest(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags,
+                                                    const double* __restrict__ rA, const double* __restrict__ rB,
+                                                    Pair<S>* __restrict__ fs) {
+    using V = V2<R>;
+    __shared__ V ring[4][kR3P];
+    const int tx = threadIdx.x, ty = threadIdx.y, t = ty * kR3X + tx;
+    const int x0 = blockIdx.x * kR3X, y0 = blockIdx.y * kR3Y, x = x0 + tx, y = y0 + ty;
+    const int z0 = blockIdx.z * kR3Z, z1 = min(z0 + kR3Z, g.nz);
+    const bool active = x < g.nx && y < g.ny;
+    const long long nxy = (long long)g.nx * g.ny;
+    int hoff[kR3N];  // in-plane offsets of this thread's halo sites
+#pragma unroll
+    for (int k = 0; k < kR3N; ++k) {
+        const int j = t + k * kR3T;
+        const int hx = x0 - 1 + j % kR3HX, hy = y0 - 1 + j / kR3HX;
+        hoff[k] = j < kR3P ? ((hy + g.ny) % g.ny) * g.nx + (hx + g.nx) % g.nx : -1;
+    }
+    double nA[kR3N], nB[kR3N];  // densities of the plane about to enter the ring
+    auto load = [&](int z) {
+        const long long o = (long long)wrapc(z, g.nz) * nxy;
+#pragma unroll
+        for (int k = 0; k < kR3N; ++k)
+            if (hoff[k] >= 0) {
+                nA[k] = rA[o + hoff[k]];
+                nB[k] = rB[o + hoff[k]];
+            }
+    };
+    auto put = [&](int z) {
+#pragma unroll
+        for (int k = 0; k < kR3N; ++k)
+            if (hoff[k] >= 0) ring[(z + 4) & 3][t + k * kR3T] = V{(R)(w19(7) * nA[k]), (R)(w19(7) * nB[k])};
+    };
+    const R lim = sizeof(R) == 8 ? (R)1e-290 : (R)1e-30;
+    auto tiny = [&](R q) { return q != (R)0 && q < lim && q > -lim; };
+    load(z0 - 1);
+    put(z0 - 1);
+    load(z0);
+    put(z0);
+    load(z0 + 1);
+    const int c0 = (ty + 1) * kR3HX + tx + 1;
+    for (int z = z0; z < z1; ++z) {
+        put(z + 1);
+        if (z + 1 < z1) load(z + 2);
+        __syncthreads();
+        if (!active) continue;
+        const long long s = (long long)z * nxy + (long long)y * g.nx + x;
+        const uint32_t fl = flags[s];
+        if (fl & k3Solid) {
+#pragma unroll
+            for (int i = 0; i < 19; ++i) store_pair<S, R>(fs + (long long)i * g.N + s, (R)0, (R)0);
+            continue;
+        }
+        st3<S, R>(fs + s, V{(R)(w19(0) * rA[s]), (R)(w19(0) * rB[s])}, P, 0);
+        const V own = ring[(z + 4) & 3][c0];
+#pragma unroll
+        for (int i = 1; i < 19; ++i) {
+            const bool bl = (fl >> (opp3(i) - 1)) & 1u;
+            const V q = bl ? own : ring[(z + e3z(i) + 4) & 3][c0 + e3y(i) * kR3HX + e3x(i)];
+            const R up = (R)(i <= 6 ? 2 : 1);
+            V v{q.x * up, q.y * up};
+            if (i <= 6 && (tiny(q.x) || tiny(q.y))) {
+                const long long n = bl ? s : site(g, x + e3x(i), y + e3y(i), z + e3z(i));
+                v = V{(R)(w19(i) * rA[n]), (R)(w19(i) * rB[n])};
+            }
+            st3<S, R>(fs + (long long)i * g.N + s, v, P, i);
+        }
     }
 }
 
@@ -1066,7 +1114,9 @@ cudaError_t set_state3(lbm3d_ctx* c, const double* f, int buf) {
 cudaError_t set_rest3(lbm3d_ctx* c, const double* a, const double* b) {
     return with_types3(c->storage, [&](auto* s_, auto* r_) {
         TYPES3(s_, r_);
-        k3_set_rest<S, R><<<grid3(c->g), kBlock3, 0, c->stream>>>(c->g, p3_of<R>(c), c->flags, a, b, state3<S>(c, c->cur));
+        const dim3 gr((unsigned)((c->g.nx + kR3X - 1) / kR3X), (unsigned)((c->g.ny + kR3Y - 1) / kR3Y),
+                      (unsigned)((c->g.nz + kR3Z - 1) / kR3Z));
+        k3_set_rest<S, R><<<gr, dim3(kR3X, kR3Y), 0, c->stream>>>(c->g, p3_of<R>(c), c->flags, a, b, state3<S>(c, c->cur));
         return cudaGetLastError();
     });
 }
@@ -1205,19 +1255,13 @@ extern "C" lbm_status lbm3d_create(const lbm3d_grid* grid, const uint8_t* solid,
     STEP3(cudaMemcpy(c->solid, solid, N, cudaMemcpyHostToDevice), "mask upload");
     k3_flags<<<gr, kBlock3, 0, c->stream>>>(c->g, c->solid, c->flags);
     STEP3(cudaGetLastError(), "flags kernel");
-    STEP3(scratch_for(c), "transfer scratch");
-    STEP3(cudaMemcpyAsync(c->scratch + 36 * N, rA0, N * sizeof(double), cudaMemcpyHostToDevice, c->stream), "density upload");
-    STEP3(cudaMemcpyAsync(c->scratch + 37 * N, rB0, N * sizeof(double), cudaMemcpyHostToDevice, c->stream), "density upload");
-    STEP3(cudaStreamSynchronize(c->stream), "upload");
-    // f = f^eq(rho, 0) into scratch [0, 38 N) -- the densities sit in its last two planes and are
-    // read before planes 36, 37 are overwritten by the same thread
-    k3_feq<double><<<gr, kBlock3, 0, c->stream>>>(c->g, c->solid, c->scratch + 36 * N, c->scratch + 37 * N, c->scratch);
-    STEP3(cudaGetLastError(), "init kernel");
-    STEP3(set_state3(c, c->scratch, 0), "init kernel");
-    STEP3(cudaGetLastError(), "init kernel");
+    STEP3(cudaMalloc(&c->dens, (size_t)2 * N * sizeof(double)), "density buffer");
+    STEP3(cudaMemcpyAsync(c->dens, rA0, N * sizeof(double), cudaMemcpyHostToDevice, c->stream), "density upload");
+    STEP3(cudaMemcpyAsync(c->dens + N, rB0, N * sizeof(double), cudaMemcpyHostToDevice, c->stream), "density upload");
+    STEP3(set_rest3(c, c->dens, c->dens + N), "init kernel");
     STEP3(cudaStreamSynchronize(c->stream), "initialisation");
-    cudaFree(c->scratch);  // transfers allocate it again on demand
-    c->scratch = nullptr;
+    cudaFree(c->dens);  // lbm3d_set_densities from host arrays allocates it again on demand
+    c->dens = nullptr;
 #undef STEP3
     *out = c;
     return LBM_OK;

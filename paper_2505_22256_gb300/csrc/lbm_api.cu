@@ -565,8 +565,7 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
         const long long N = (long long)c.hcases[i].nx * c.hcases[i].ny;
         STEP(cudaMemcpyAsync(c.fields, cs[i].rho_A0, N * sizeof(double), cudaMemcpyHostToDevice, c.stream), "density upload");
         STEP(cudaMemcpyAsync(c.fields + N, cs[i].rho_B0, N * sizeof(double), cudaMemcpyHostToDevice, c.stream), "density upload");
-        STEP(launch_feq_rest(c, i, c.fields, c.fields + N, c.dense), "init kernel");
-        STEP(launch_set_state(c, i, c.dense), "init kernel");
+        STEP(launch_set_rest(c, i, c.fields, c.fields + N), "init kernel");
     }
     STEP(cudaStreamSynchronize(c.stream), "initialisation");
 #undef STEP
@@ -692,8 +691,7 @@ lbm_status lbm_set_densities(lbm_ctx* ctx, int32_t ci, const double* rho_A0, con
         a = c.fields;
         b = c.fields + N;
     }
-    CUDA_TRY(launch_feq_rest(c, ci, a, b, c.dense));
-    CUDA_TRY(launch_set_state(c, ci, c.dense));
+    CUDA_TRY(launch_set_rest(c, ci, a, b));
     ++c.version;
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(c.stream));
     return LBM_OK;

@@ -235,59 +235,117 @@ __global__ void k_wall_scatter(const DevCase* __restrict__ cases, int c, const i
     }
 }
 
-// f = f^eq(rho_k, 0) in every case at once (cases along blockIdx.y): the stored populations that
-// k_feq_rest followed by k_set_state write, computed straight from the densities (all cases back to
-// back, case c at d_off) with the same double-precision products, so the state is the same bit for
-// bit.  The stored f*_i at x is what the next pull takes: w_i rho(x + e_i) from a fluid neighbour,
-// w_i rho(x) across a blocked link or beyond an open edge (the outlet column's own value where the
-// copy rule keeps it); G ghost columns repeat the periodic edges.
+// ------------------------------------------------------------------------------------------------
+// f = f^eq(rho_k, 0) in the listed cases (along blockIdx.y), straight from the densities (case c at
+// d_off - base).  The stored f*_i at x is what the next pull takes: w_i rho(x + e_i) from a fluid
+// neighbour, w_i rho(x) across a blocked link or beyond an open edge (the outlet column's own value
+// where the copy rule keeps it), minus w_i rho0 in 16-bit storage; G ghost columns repeat the
+// periodic edges.
+//
+// The value is (R)(w_i rho - w_i rho0) with FP64 products.  4/9, 1/9 and 1/36 in FP64 are powers of
+// two apart, so every direction's product, shift and rounding is an exact power of two times that of
+// q = (R)(rho / 36 - rho0 / 36): one FP64 product and conversion per node and component instead of
+// nine, the same bits.  (GB300 issues two FP64 operations per SM and cycle: at 36 of them per node the
+// pass ran at the FP64 pipe's rate, 458 us on seven 1024 x 1024 FP32 cases where its 88 B per node
+// take 95 us of HBM time; now 150 us, most of it its stores.)  A q so small that scaling it up
+// could differ from rounding the larger product takes the direct form.
+//
+// A block of kRestT columns (one halo column on each side) marches down kRestRows rows; q of the row
+// ahead goes into a ring of four shared-memory rows, one barrier per row.
+// ------------------------------------------------------------------------------------------------
+constexpr int kRestT = 128, kRestW = kRestT - 2, kRestRows = 16;
+
+template <class R>
+__device__ __forceinline__ bool rest_tiny(R q) {  // nonzero and near the denormals of R
+    const R lim = sizeof(R) == 8 ? (R)1e-290 : (R)1e-30;
+    return q != (R)0 && q < lim && q > -lim;
+}
+
 template <class S>
-__global__ void k_set_rest_all(const DevCase* __restrict__ cases, int G, const uint8_t* __restrict__ solid_all,
-                               const uint16_t* __restrict__ flags_all, const double* __restrict__ rhoA_all,
-                               const double* __restrict__ rhoB_all, Pair<S>* __restrict__ out_all) {
+__global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__ cases, int G, long long base,
+                                                     const uint8_t* __restrict__ solid_all,
+                                                     const uint16_t* __restrict__ flags_all,
+                                                     const double* __restrict__ rhoA_all,
+                                                     const double* __restrict__ rhoB_all, Pair<S>* __restrict__ out_all) {
     using R = typename ComputeOf<S>::type;
-    const DevCase C = cases[blockIdx.y];
-    const long long N = (long long)C.nx * C.ny;
-    const long long plane = C.pitch;
-    Pair<S>* out = out_all + C.f_off;
-    const double* rk[2] = {rhoA_all + C.d_off, rhoB_all + C.d_off};
+    using V = V2<R>;
+    __shared__ V ring[4][kRestT];
+    const DevCase& C = cases[blockIdx.y];
+    const int nx = C.nx, ny = C.ny, bcx = C.bc_x, t = threadIdx.x;
+    const int nstrip = (nx + kRestW - 1) / kRestW;
+    const int chunk = blockIdx.x / nstrip, xs = (blockIdx.x % nstrip) * kRestW;
+    const int y0 = chunk * kRestRows, y1 = min(y0 + kRestRows, ny);
+    if (y0 >= ny) return;  // the grid covers the case with the most tiles
+    const long long plane = C.pitch, row = 9 * plane;
+    const double* rA = rhoA_all + (C.d_off - base);
+    const double* rB = rhoB_all + (C.d_off - base);
     const uint8_t* sol = solid_all + C.d_off;
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N; s += (long long)gridDim.x * blockDim.x) {
-        const int X = (int)(s % C.nx), Y = (int)(s / C.nx);
-        const uint16_t fl = flags_all[C.d_off + s];
-        const long long o = (long long)Y * 9 * C.pitch + X + G;
-        R ov[2][9];
-        for (int k = 0; k < 2; ++k) {
+    const uint16_t* flags = flags_all + C.d_off;
+    Pair<S>* out = out_all + C.f_off;
+    const double sh[2] = {wq(5) * C.rho0[0], wq(5) * C.rho0[1]};
+    const int x = xs - 1 + t;  // window column
+    int X = x;                 // its lattice column, -1 outside a closed or open edge (never pulled from)
+    if (x < 0 || x >= nx) X = bcx != kPeriodic ? -1 : (x < 0 ? x + nx : x % nx);
+    const bool mine = t >= 1 && t <= kRestW && x < nx;
+
+    auto scaled = [&](double r, int k) -> double {
+        double v = wq(5) * r;
+        if constexpr (Store<S>::kShift) v -= sh[k];
+        return v;
+    };
+    double nA = 0.0, nB = 0.0;  // densities of the row about to enter the ring
+    auto load = [&](int r) {
+        nA = nB = 0.0;
+        if (r < 0 || r >= ny) {
+            if (C.bc_y != kPeriodic) return;
+            r += r < 0 ? ny : -ny;
+        }
+        if (X < 0) return;
+        const long long s = (long long)r * nx + X;
+        if (sol[s]) return;
+        nA = rA[s];
+        nB = rB[s];
+    };
+    auto put = [&](int r) { ring[r & 3][t] = V{(R)scaled(nA, 0), (R)scaled(nB, 1)}; };
+    load(y0 - 1);
+    put(y0 - 1);
+    load(y0);
+    put(y0);
+    load(y0 + 1);
+    for (int y = y0; y < y1; ++y) {
+        put(y + 1);
+        if (y + 1 < y1) load(y + 2);
+        __syncthreads();
+        if (mine) {
+            const long long s = (long long)y * nx + x;
+            const uint16_t fl = flags[s];
+            const bool solid = (fl & kSolidBit) != 0;
+            Pair<S>* o = out + y * row + x + G;
+            const bool gr = bcx == kPeriodic && x < G, gl = bcx == kPeriodic && x >= nx - G;  // ghost copies
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                double v = 0.0;
-                if (!(fl & kSolidBit)) {
-                    int tx = X + cx(i), ty = Y + cy(i);
-                    long long src = s;
-                    int q = i;
-                    if (C.bc_x == kOpen && (tx < 0 || tx >= C.nx)) {
-                        q = (X == C.nx - 1 && (fl & kOutletOwnBit) && cx(i) > 0) ? opp(i) : i;
-                    } else if (i != 0 && ((fl >> (opp(i) - 1)) & 1u)) {
-                        q = opp(i);
-                    } else {
-                        tx += (tx < 0) ? C.nx : 0;
-                        tx -= (tx >= C.nx) ? C.nx : 0;
-                        ty += (ty < 0) ? C.ny : 0;
-                        ty -= (ty >= C.ny) ? C.ny : 0;
-                        src = (long long)ty * C.nx + tx;
+                const bool edge = bcx == kOpen && (x + cx(i) < 0 || x + cx(i) >= nx);
+                const bool own = i == 0 || edge || ((fl >> (opp(i) - 1)) & 1u);
+                const V q = own ? ring[y & 3][t] : ring[(y + cy(i)) & 3][t + cx(i)];
+                const R up = (R)(i == 0 ? 16 : (i <= 4 ? 4 : 1));
+                V v{q.x * up, q.y * up};
+                if (rest_tiny(q.x) || rest_tiny(q.y)) {
+                    int tx = x, ty = y;
+                    if (!own) {
+                        tx += cx(i);
+                        ty += cy(i);
+                        tx += tx < 0 ? nx : (tx >= nx ? -nx : 0);
+                        ty += ty < 0 ? ny : (ty >= ny ? -ny : 0);
                     }
-                    v = wq(q) * (sol[src] ? 0.0 : rk[k][src]);  // the value k_feq_rest holds at src
-                    if constexpr (Store<S>::kShift) v -= wq(i) * C.rho0[k];
+                    const long long z = (long long)ty * nx + tx;
+                    v = sol[z] ? V{(R)0, (R)0}
+                               : V{(R)(scaled(rA[z], 0) * (double)up), (R)(scaled(rB[z], 1) * (double)up)};
                 }
-                ov[k][i] = (R)v;
+                if (solid) v = V{(R)0, (R)0};
+                store_pair<S, R>(o + i * plane, v.x, v.y);
+                if (gr) store_pair<S, R>(o + i * plane + nx, v.x, v.y);
+                if (gl) store_pair<S, R>(o + i * plane - nx, v.x, v.y);
             }
-        }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            Pair<S>* p = out + i * plane;
-            store_pair<S, R>(p + o, ov[0][i], ov[1][i]);
-            if (C.bc_x == kPeriodic && X < G) store_pair<S, R>(p + o + C.nx, ov[0][i], ov[1][i]);
-            if (C.bc_x == kPeriodic && X >= C.nx - G) store_pair<S, R>(p + o - C.nx, ov[0][i], ov[1][i]);
         }
     }
 }
@@ -332,27 +390,37 @@ cudaError_t launch_wall_cast(Ctx& c, int ci) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_set_rest_all(Ctx& c, const double* rhoA_all, const double* rhoB_all) {
-    long long nmax = 0;
-    for (const auto& h : c.hcases) nmax = nmax > (long long)h.nx * h.ny ? nmax : (long long)h.nx * h.ny;
-    const int nc = (int)c.hcases.size(), G = ghost_cols(c.storage);
-    for (int c0 = 0; c0 < nc; c0 += 65535) {  // cases along gridDim.y, at most 65535 per launch
-        const int n = nc - c0 < 65535 ? nc - c0 : 65535;
-        // about 4,096 blocks in all, at least one per case
-        long long bx = ((nmax + 255) / 256 < 4096 ? (nmax + 255) / 256 : 4096);
-        bx = bx * 8 / n > 0 ? (bx * 8 / n < bx ? bx * 8 / n : bx) : 1;
-        const dim3 g((unsigned)bx, (unsigned)n);
+// cases [c0, c0 + n) with the densities of case c at d_off - base
+static cudaError_t set_rest_cases(Ctx& c, int c0, int n, long long base, const double* rhoA, const double* rhoB) {
+    const int G = ghost_cols(c.storage);
+    for (const int end = c0 + n; c0 < end; c0 += 65535) {  // cases along gridDim.y, at most 65535 per launch
+        const int m = end - c0 < 65535 ? end - c0 : 65535;
+        long long tiles = 1;
+        for (int i = c0; i < c0 + m; ++i) {
+            const DevCase& h = c.hcases[i];
+            const long long k = (long long)((h.nx + kRestW - 1) / kRestW) * ((h.ny + kRestRows - 1) / kRestRows);
+            tiles = tiles > k ? tiles : k;
+        }
+        const dim3 g((unsigned)tiles, (unsigned)m);
         const DevCase* dc = c.dcases + c0;
         switch (c.storage) {
-            case LBM_STORE_F64: k_set_rest_all<double><<<g, 256, 0, c.stream>>>(dc, G, c.solid, c.flags, rhoA_all, rhoB_all, (Pair<double>*)c.f[c.cur]); break;
-            case LBM_STORE_F32: k_set_rest_all<float><<<g, 256, 0, c.stream>>>(dc, G, c.solid, c.flags, rhoA_all, rhoB_all, (Pair<float>*)c.f[c.cur]); break;
-            case LBM_STORE_F16_SHIFTED: k_set_rest_all<__half><<<g, 256, 0, c.stream>>>(dc, G, c.solid, c.flags, rhoA_all, rhoB_all, (Pair<__half>*)c.f[c.cur]); break;
-            default: k_set_rest_all<__nv_bfloat16><<<g, 256, 0, c.stream>>>(dc, G, c.solid, c.flags, rhoA_all, rhoB_all, (Pair<__nv_bfloat16>*)c.f[c.cur]); break;
+            case LBM_STORE_F64: k_set_rest<double><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<double>*)c.f[c.cur]); break;
+            case LBM_STORE_F32: k_set_rest<float><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<float>*)c.f[c.cur]); break;
+            case LBM_STORE_F16_SHIFTED: k_set_rest<__half><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<__half>*)c.f[c.cur]); break;
+            default: k_set_rest<__nv_bfloat16><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<__nv_bfloat16>*)c.f[c.cur]); break;
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_set_rest_all(Ctx& c, const double* rhoA_all, const double* rhoB_all) {
+    return set_rest_cases(c, 0, (int)c.hcases.size(), 0, rhoA_all, rhoB_all);
+}
+
+cudaError_t launch_set_rest(Ctx& c, int ci, const double* rhoA, const double* rhoB) {
+    return set_rest_cases(c, ci, 1, c.hcases[ci].d_off, rhoA, rhoB);
 }
 
 }  // namespace lbm

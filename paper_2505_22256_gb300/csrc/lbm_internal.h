@@ -131,8 +131,9 @@ cudaError_t launch_densities_all(Ctx& c, double* rhoA_all, double* rhoB_all);
 cudaError_t launch_set_state(Ctx& c, int case_index, const double* dense_f);
 // f = f^eq(rho_k, 0) in every case from densities of all cases back to back (one launch per 65,535 cases)
 cudaError_t launch_set_rest_all(Ctx& c, const double* rhoA_all, const double* rhoB_all);
+// the same for one case, whose densities start at rhoA / rhoB
+cudaError_t launch_set_rest(Ctx& c, int case_index, const double* rhoA, const double* rhoB);
 cudaError_t launch_get_state(Ctx& c, int case_index, double* dense_f);
-cudaError_t launch_feq_rest(Ctx& c, int case_index, const double* rhoA, const double* rhoB, double* dense_f);
 int step_smem_bytes(int storage, int threads);
 cudaError_t step_occupancy(int storage, int threads, int* blocks_per_sm);
 int ghost_cols(int storage);      // ghost columns on each side of a stored population row

@@ -848,22 +848,6 @@ __global__ void k_sliding_walls(const DevCase* __restrict__ cases, const int* __
 // ------------------------------------------------------------------------------------------------
 // State transfer kernels (dense doubles [2][9][ny][nx] <-> the post-collision buffer)
 // ------------------------------------------------------------------------------------------------
-__global__ void k_feq_rest(const DevCase* __restrict__ cases, int c, const uint8_t* __restrict__ solid_all,
-                           const double* __restrict__ rhoA, const double* __restrict__ rhoB,
-                           double* __restrict__ f) {
-    const DevCase C = cases[c];
-    const long long N = (long long)C.nx * C.ny;
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < N; s += (long long)gridDim.x * blockDim.x) {
-        const bool sol = solid_all[C.d_off + s] != 0;
-        const double a = sol ? 0.0 : rhoA[s], b = sol ? 0.0 : rhoB[s];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            f[(long long)i * N + s] = wq(i) * a;
-            f[(long long)(9 + i) * N + s] = wq(i) * b;
-        }
-    }
-}
-
 // Post-streaming populations -> post-collision buffer: the inverse of the pull, so that the next
 // pull reproduces f exactly (up to the storage rounding).  Ghost columns are filled as well.
 template <class S>
@@ -1149,12 +1133,6 @@ cudaError_t launch_diag_all(Ctx& c, double* rhoA_all, double* rhoB_all) {
     cudaError_t e = dispatch(c, a, c.stream, true, grid);
     if (e != cudaSuccess) return e;
     k_diag_reduce<<<(unsigned)c.hcases.size(), 32, 0, c.stream>>>(c.dcases, -1, c.diag_part, c.diag_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_feq_rest(Ctx& c, int ci, const double* rhoA, const double* rhoB, double* dense_f) {
-    const long long N = (long long)c.hcases[ci].nx * c.hcases[ci].ny;
-    k_feq_rest<<<blocks_for(N), 256, 0, c.stream>>>(c.dcases, ci, c.solid, rhoA, rhoB, dense_f);
     return cudaGetLastError();
 }
 
