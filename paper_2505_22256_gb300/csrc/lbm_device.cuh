@@ -298,6 +298,36 @@ __device__ __forceinline__ V2<R> vbc(T v) {  // the same value in both lanes, in
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
+// ------------------------------------------------------------------------------------------------
+// Programmatic dependent launch.  A step is one short launch behind another: a kernel launched with
+// PdlLaunch may become resident while the launch before it drains, and runs its setup (barriers, work
+// item, parameters) there.  pdl_wait() returns once every launch before it has completed and its
+// writes are visible; nothing those launches write or read may be touched before it.
+// pdl_launch_next() lets the launch after this one start the same way; it comes after the wait, so
+// at most one launch waits behind the running one.  Per step this takes 1 to 3 us (the gap between
+// launches and the setup): 96 x 96 in one-row items 7.3 -> 6.3 us, 350 x 150 open channel 28.6 ->
+// 25.7 us, seven 1024 x 1024 cases 185 -> 182.5 us, with the sliding-wall pass 20.0 -> 18.9 us.
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+struct PdlLaunch {
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg;
+    PdlLaunch(dim3 grid, dim3 block, size_t smem, cudaStream_t s) : attr(), cfg() {
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+    }
+    PdlLaunch(const PdlLaunch&) = delete;
+    PdlLaunch& operator=(const PdlLaunch&) = delete;
+};
+
 // Compute type for a storage type: FP64 storage computes in FP64, everything else in FP32.
 template <class S>
 struct ComputeOf {

@@ -454,7 +454,6 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
         fence_mbar_init();
         fence_proxy_async_smem();
     }
-    __syncthreads();
 
     // Row loads are numbered per block: load n goes to slot n % kSlots and completes phase
     // n / kSlots of that slot's barrier.  (slot, parity) of the next load to issue and of the next
@@ -466,19 +465,23 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
     uint32_t so_m = 0, so_0 = 0, so_p = 0;
     bool failed = false;
 
-    // Work items are claimed from a counter, so blocks that share a busy SM take fewer of them.  The
-    // claiming thread also copies the item's case parameters to shared memory: the rarely used ones
-    // (adhesion, inlet) are read from there where needed instead of occupying registers.
+    // Work items: block b starts with item b and claims the later ones from a counter, so blocks that
+    // share a busy SM take fewer of them.  The block copies the item's case parameters to shared
+    // memory: the rarely used ones (adhesion, inlet) are read from there where needed instead of
+    // occupying registers.
     __shared__ int s_claim;
-    __shared__ Params<R> s_par;
-    auto claim = [&]() {
-        const int k = atomicAdd(a.sched, 1);
-        s_claim = k;
-        if (a.item_begin + k < a.item_end) s_par = load_params<R>(a.cases[a.items[a.item_begin + k].x & 0x7FFFFFFF]);
+    __shared__ __align__(8) Params<R> s_par;
+    auto copy_params = [&](int it) {
+        const int* src = reinterpret_cast<const int*>(&case_params<R>(a.cases[a.items[it].x & 0x7FFFFFFF]));
+        for (int w = t; w < (int)(sizeof(Params<R>) / sizeof(int)); w += T) reinterpret_cast<int*>(&s_par)[w] = src[w];
     };
-    if (t == 0) claim();
+    int it = a.item_begin + (int)blockIdx.x;
+    if (it < a.item_end) copy_params(it);
+    // everything above reads only what no kernel writes; the state, the counters and the outputs may
+    // still be in use by the launch before this one
+    pdl_wait();
+    pdl_launch_next();
     __syncthreads();
-    int it = a.item_begin + s_claim;
     while (it < a.item_end) {
         const int4 item = a.items[it];
         const int ci = item.x & 0x7FFFFFFF;       // case
@@ -773,9 +776,11 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
             }
             __syncthreads();
         }
-        if (t == 0) claim();  // every thread is past the previous claim and its parameters
+        if (t == 0) s_claim = a.item_begin + (int)gridDim.x + atomicAdd(a.sched, 1);
+        __syncthreads();  // every thread is past the previous item's parameters, too
+        it = s_claim;
+        if (it < a.item_end) copy_params(it);
         __syncthreads();
-        it = a.item_begin + s_claim;
     }
     if (t == 0) {
         // the last block to finish sees every claim made and resets the counters for the next launch
@@ -808,6 +813,8 @@ __global__ void k_sliding_walls(const DevCase* __restrict__ cases, const int* __
                                 const uint16_t* __restrict__ flags_all, Pair<S>* __restrict__ buf_all) {
     using R = typename ComputeOf<S>::type;
     constexpr int G = Layout<S>::G;
+    pdl_wait();
+    pdl_launch_next();
     const int ci = list[blockIdx.y >> 1];
     const bool upper = blockIdx.y & 1;
     const DevCase& C = cases[ci];
@@ -1019,11 +1026,10 @@ StepArgs make_args(Ctx& c, int ib, int ie, double* o4[4], double* part) {
 template <class S, int T>
 cudaError_t launch_step_w(const Ctx& c, const StepArgs& a, cudaStream_t s, bool fields, int grid) {
     using R = typename ComputeOf<S>::type;
-    const size_t smem = smem_for<S>(T);
-    if (fields) k_step<S, R, true, false, T><<<grid, T, smem, s>>>(a);
-    else if (c.wall_inline) k_step<S, R, false, true, T><<<grid, T, smem, s>>>(a);
-    else k_step<S, R, false, false, T><<<grid, T, smem, s>>>(a);
-    return cudaGetLastError();
+    const PdlLaunch l(dim3((unsigned)grid), dim3(T), smem_for<S>(T), s);
+    if (fields) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, true, false, T>, a);
+    if (c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, false, true, T>, a);
+    return cudaLaunchKernelEx(&l.cfg, k_step<S, R, false, false, T>, a);
 }
 
 template <class S>
@@ -1040,6 +1046,12 @@ cudaError_t dispatch(Ctx& c, const StepArgs& a, cudaStream_t s, bool fields, int
         case LBM_STORE_F16_SHIFTED: return launch_step_t<__half>(c, a, s, fields, grid);
         default: return launch_step_t<__nv_bfloat16>(c, a, s, fields, grid);
     }
+}
+
+template <class S>
+cudaError_t launch_slide(const PdlLaunch& l, const Ctx& c, void* fout) {
+    return cudaLaunchKernelEx(&l.cfg, k_sliding_walls<S>, (const DevCase*)c.dcases, (const int*)c.slide_list,
+                              (const uint16_t*)c.flags, (Pair<S>*)fout);
 }
 
 int blocks_for(long long n) { return (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096); }
@@ -1084,14 +1096,13 @@ cudaError_t launch_step(Ctx& c, int in_buf, cudaStream_t s) {
     a.fout = c.f[1 - in_buf];
     cudaError_t e = dispatch(c, a, s, false, c.grid_blocks);
     if (e != cudaSuccess || c.slide_n == 0) return e;
-    const dim3 grid((unsigned)((c.slide_max_nx + 127) / 128), (unsigned)(2 * c.slide_n));
+    const PdlLaunch l(dim3((unsigned)((c.slide_max_nx + 127) / 128), (unsigned)(2 * c.slide_n)), dim3(128), 0, s);
     switch (c.storage) {
-        case LBM_STORE_F64: k_sliding_walls<double><<<grid, 128, 0, s>>>(c.dcases, c.slide_list, c.flags, (Pair<double>*)a.fout); break;
-        case LBM_STORE_F32: k_sliding_walls<float><<<grid, 128, 0, s>>>(c.dcases, c.slide_list, c.flags, (Pair<float>*)a.fout); break;
-        case LBM_STORE_F16_SHIFTED: k_sliding_walls<__half><<<grid, 128, 0, s>>>(c.dcases, c.slide_list, c.flags, (Pair<__half>*)a.fout); break;
-        default: k_sliding_walls<__nv_bfloat16><<<grid, 128, 0, s>>>(c.dcases, c.slide_list, c.flags, (Pair<__nv_bfloat16>*)a.fout); break;
+        case LBM_STORE_F64: return launch_slide<double>(l, c, a.fout);
+        case LBM_STORE_F32: return launch_slide<float>(l, c, a.fout);
+        case LBM_STORE_F16_SHIFTED: return launch_slide<__half>(l, c, a.fout);
+        default: return launch_slide<__nv_bfloat16>(l, c, a.fout);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_fields(Ctx& c, int ci, double* rhoA, double* rhoB, double* ux, double* uy, bool diag) {
