@@ -479,9 +479,9 @@ def run_reference(args):
 # ------------------------------------------------------------------------------------------------
 # our arm
 # ------------------------------------------------------------------------------------------------
-# the candidates of lbm_autotune: wall-list form, block width, row chunks (0 guided, < 0 guided with
+# the candidates of lbm_autotune: wall-list form, block width, row chunks (0 automatic, < 0 guided with
 # short tail items, > 0 uniform)
-LAUNCH_SHAPES = [(w, t, r) for w in (0, 1) for t in (128, 64) for r in (0, -8, 16, 32, 64, 128)]
+LAUNCH_SHAPES = [(w, t, r) for w in (0, 1) for t in (128, 64) for r in (0, -8, -16, 16, 32, 64, 128)]
 
 
 def launch_table(args, lat, stream) -> int:

@@ -336,9 +336,10 @@ lbm_status lbm_info(lbm_ctx* ctx, lbm_info_t* out);
 /* Set the step kernel's launch shape: threads per block (128 or 64, the widths the kernel is built
  * for; a work item spans that many columns minus 8 halo columns; lbm_create picks the width that
  * launches fewer thread columns over all cases) and rows per work item: >= 1 for uniform items of
- * that height, or 0 (the default) for a guided list -- long items first, then 16-row items that
+ * that height; -64 .. -1 for a guided list -- long items first, then items of -block_rows rows that
  * even out the end of the launch, the long height chosen to balance the list over the resident
- * blocks; -64 .. -1 for a guided list whose short items have -block_rows rows.  Rebuilds the work
+ * blocks; or 0 (the default) for the library's choice: a guided list with 8- or 16-row short items, or
+ * short uniform items where those spread a small lattice over more of the GPU.  Rebuilds the work
  * list and drops the captured graph.  LBM_EINVAL for other widths or block_rows < -64. */
 lbm_status lbm_set_launch(lbm_ctx* ctx, int32_t block_threads, int32_t block_rows);
 
@@ -354,13 +355,13 @@ lbm_status lbm_selftest_wait_timeout(lbm_ctx* ctx, double limit_ms);
 
 /* Choose the step kernel's form for wall-list nodes (the second-layer correction of Table 1): 1
  * inlines it (faster where wall-list nodes are common, e.g. porous media), 0 calls an out-of-line
- * copy (keeps the loop of warps without wall-list nodes small).  lbm_create picks 1 when wall-list
- * nodes exceed 4 % of the fluid nodes; lbm_autotune tries both.  Results agree to FP rounding.
+ * copy.  lbm_create picks 1 when wall-list nodes exceed 4 % of the fluid nodes or the cases hold more
+ * than 2^18 nodes; lbm_autotune tries both.  Results agree to FP rounding.
  * Drops the captured graph.  LBM_EINVAL for other values. */
 lbm_status lbm_set_wall_path(lbm_ctx* ctx, int32_t inline_correction);
 
 /* Time candidate launch shapes on the live state (the current shape first, then both widths x both
- * wall-list forms x the row settings 0, -8, 16, 32, 64, 128; each twice for `steps` steps after one
+ * wall-list forms x the row settings 0, -8, -16, 16, 32, 64, 128; each twice for `steps` steps after one
  * warm-up launch, keeping the faster time) and keep the fastest; a shape replaces the best so far
  * only when it is at least 1 % faster, so that shapes within the timing noise do not trade places
  * from run to run.  The state advances by the steps taken; best_ms (may be NULL)

@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <chrono>
 #include <string>
 #include <thread>
@@ -232,32 +233,52 @@ lbm_status build_tmaps(Ctx& c) {
     return LBM_OK;
 }
 
-#ifndef LBM_TAIL_ROWS
-#define LBM_TAIL_ROWS 16  // height of the short items that end a launch
-#endif
+// What a launch of the step kernel costs, in rows marched by a block that has its SM to itself (about
+// 0.9 us in FP32, 1.1 in 16-bit storage, 10.7 in FP64, where the FP64 pipe sets the pace).  An item
+// costs its rows plus `fill` (halo rows, first loads).  Blocks that share an SM slow each other by
+// `shared` while the state stays in L2 and by `spilled` when it does not; `full` scales the guided
+// list's estimate, which counts its last short item whole, to the same unit.  Fitted to uniform lists of 1- to 32-row items on fifteen lattices.
+struct RowCost {
+    double fill, shared, spilled, full;
+};
+RowCost row_cost(int storage) {
+    if (storage == LBM_STORE_F64) return {1.3, 2.0, 2.0, 1.8};
+    return storage == LBM_STORE_F32 ? RowCost{4.5, 1.3, 1.6, 0.92} : RowCost{4.5, 1.5, 1.7, 0.92};
+}
+// n items of h rows that are all resident at once; blocks: items per SM, in blocks of 128 threads
+double one_round_cost(const RowCost& m, double blocks, int h, bool in_l2) {
+    return (h + m.fill) * (blocks <= 1.0 ? 1.0 : (in_l2 ? m.shared : m.spilled));
+}
 
 // Row chunks [y0, y1) of one case's column strips, chunk-major; odd chunks march upwards (sign bit
 // of the case field), so the halo rows two neighbouring chunks share are read at about the same
 // time, while they are still in L2.
-void push_chunks(std::vector<int4>& out, int ci, int nstrip, int Wi, int y_begin, int y_end, int h) {
+// alternate = false: every chunk marches down the rows, so the gradient sums of a row (formed in
+// marching order) do not depend on the chunk heights.
+void push_chunks(std::vector<int4>& out, int ci, int nstrip, int Wi, int y_begin, int y_end, int h, bool alternate = true) {
     const int n = (y_end - y_begin + h - 1) / h;
     for (int k = 0; k < n; ++k) {
         // balanced heights: the first (rows % n) chunks take one row more
         const int rows = y_end - y_begin, base = rows / n, extra = rows % n;
         const int y0 = y_begin + k * base + std::min(k, extra), y1 = y0 + base + (k < extra ? 1 : 0);
         for (int s = 0; s < nstrip; ++s)
-            out.push_back(make_int4((int)((unsigned)ci | ((k & 1) ? 0x80000000u : 0u)), s * Wi, y0, y1));
+            out.push_back(make_int4((int)((unsigned)ci | ((alternate && (k & 1)) ? 0x80000000u : 0u)), s * Wi, y0, y1));
     }
 }
 
 // Work lists.  A work item is a column window of block_threads - 8 interior columns by a chunk of
 // rows of one case; blocks of the step kernel claim items in list order from a counter.
-//  * Step list.  With block_rows > 0, uniform chunks of that height.  With block_rows = 0 (the
-//    default; block_rows < 0 for a tail of -block_rows rows), a guided list: long chunks of height
-//    Hb first, then short chunks of LBM_TAIL_ROWS
-//    rows, enough of them to absorb the ragged end of the long ones, so that a launch lasts about
-//    (rows marched, 5 halo rows per item included) / (resident blocks) + one short item.  Hb
-//    minimises that estimate.
+//  * Step list.  With block_rows > 0, uniform chunks of that height.  With block_rows < 0, a guided
+//    list: long chunks of height Hb first, then short chunks of -block_rows rows, enough of them to
+//    absorb the ragged end of the long ones, so that a launch lasts about (rows marched, 5 halo
+//    rows per item included) / (resident blocks) + one short item.  Hb minimises that estimate.
+//    With block_rows = 0 (the default), the cheapest by row_cost of that list with 8- and with
+//    16-row short chunks and of the uniform chunks that are all resident at once: a lattice that cannot
+//    fill the GPU in 16-row items is a serial chain of rows on a few SMs, and shorter items spread it.
+//    us per step, 16-row items -> this rule: 96 x 96 FP64 183 -> 28, FP32 19.9 -> 6.4, 350 x 150 open
+//    25.7 -> 8.0, 300 x 350 20.8 -> 10.2, four of them 26.5 -> 19.1, 512 x 512 21.5 -> 13.4, 14 of 300 x 350
+//    54.8 -> 52.7, 2048 x 512 FP16 38.0 -> 36.0.  The uniform chunks all march down, so a small case alone
+//    and the same case in a small ensemble reach the same bits at any height.
 //  * Per-case list (after the step list): uniform chunks, contiguous per case, used by the fields
 //    pass, whose per-item partial sums are reduced per case in item order.
 lbm_status build_items(Ctx& c) {
@@ -276,49 +297,88 @@ lbm_status build_items(Ctx& c) {
         strips += nstrip[i];
     }
     std::vector<int4> items;
+    const RowCost model = row_cost(c.storage);
+    auto uniform_items = [&](int h) -> long long {
+        long long n = 0;
+        for (int i = 0; i < ncases; ++i) n += (long long)nstrip[i] * ((c.hcases[i].ny + h - 1) / h);
+        return n;
+    };
+    const bool in_l2 = 2.0 * c.pop_elems * c.elem < 110e6;  // both state buffers, 129 MB of L2
+    auto uniform_cost = [&](int h) -> double {  // < 0: not resident at once
+        const long long n = uniform_items(h);
+        return n <= resident ? one_round_cost(model, (double)n * W / 128.0 / c.num_sms, h, in_l2) : -1.0;
+    };
+    // rows of short chunks (Hs) per strip of case i for a given long height hb
+    auto tail_chunks = [&](int i, int hb, int Hs) -> int {
+        const long long need = (resident * (hb + 5) + strips * (Hs + 5) - 1) / (strips * (Hs + 5));
+        return (int)std::min<long long>(need, c.hcases[i].ny / Hs);
+    };
     if (c.block_rows > 0) {
-        const int H = c.block_rows;
-        for (int i = 0; i < ncases; ++i) push_chunks(items, i, nstrip[i], Wi, 0, c.hcases[i].ny, H);
-        c.rows_used = H;
+        for (int i = 0; i < ncases; ++i) push_chunks(items, i, nstrip[i], Wi, 0, c.hcases[i].ny, c.block_rows);
+        c.rows_used = c.block_rows;
     } else {
-        const int Hs = c.block_rows < 0 ? -c.block_rows : LBM_TAIL_ROWS;
-        // rows of short chunks per strip of case i for a given long height hb
-        auto tail_chunks = [&](int i, int hb) -> int {
-            const long long need = (resident * (hb + 5) + strips * (Hs + 5) - 1) / (strips * (Hs + 5));
-            return (int)std::min<long long>(need, c.hcases[i].ny / Hs);
-        };
         double best = -1.0;
-        int Hb = 32;
-        for (int hb = 16; hb <= 256; ++hb) {
-            double work = 0.0, tail = 0.0;
+        int Hb = 32, Hs = 16;
+        for (const int hs : {16, 8}) {
+            if (c.block_rows < 0 && hs != 16) break;
+            const int short_h = c.block_rows < 0 ? -c.block_rows : hs;
+            for (int hb = 16; hb <= 256; ++hb) {
+                double work = 0.0, tail = 0.0;
+                for (int i = 0; i < ncases; ++i) {
+                    const int ns = tail_chunks(i, hb, short_h), bulk = c.hcases[i].ny - ns * short_h;
+                    const int nb = (bulk + hb - 1) / hb;
+                    work += (double)nstrip[i] * (bulk + 5.0 * nb + ns * (short_h + 5.0));
+                    tail += (double)nstrip[i] * ns * (short_h + 5.0);
+                }
+                const double cost = work / resident + (short_h + 5) + std::max(0.0, (hb + 5) - tail / resident);
+                if (best < 0 || cost < (short_h == Hs ? best : 0.997 * best)) {
+                    best = cost;
+                    Hb = hb;
+                    Hs = short_h;
+                }
+            }
+        }
+        int H = 0;
+        if (c.block_rows == 0) {
+            best *= model.full;
+            for (int h = 1; h <= 64; ++h) {
+                const double cost = uniform_cost(h);
+                if (cost >= 0 && cost < best) {
+                    best = cost;
+                    H = h;
+                }
+            }
+        }
+        if (H > 0) {
+            for (int i = 0; i < ncases; ++i) push_chunks(items, i, nstrip[i], Wi, 0, c.hcases[i].ny, H, false);
+            c.rows_used = H;
+        } else {
+            std::vector<int> ns(ncases);
             for (int i = 0; i < ncases; ++i) {
-                const int ns = tail_chunks(i, hb), bulk = c.hcases[i].ny - ns * Hs;
-                const int nb = (bulk + hb - 1) / hb;
-                work += (double)nstrip[i] * (bulk + 5.0 * nb + ns * (Hs + 5.0));
-                tail += (double)nstrip[i] * ns * (Hs + 5.0);
+                ns[i] = tail_chunks(i, Hb, Hs);
+                push_chunks(items, i, nstrip[i], Wi, 0, c.hcases[i].ny - ns[i] * Hs, Hb);
             }
-            const double cost = work / resident + (Hs + 5) + std::max(0.0, (hb + 5) - tail / resident);
-            if (best < 0 || cost < best) {
-                best = cost;
-                Hb = hb;
-            }
+            for (int i = 0; i < ncases; ++i)
+                if (ns[i] > 0) push_chunks(items, i, nstrip[i], Wi, c.hcases[i].ny - ns[i] * Hs, c.hcases[i].ny, Hs);
+            c.rows_used = Hb;
         }
-        std::vector<int> ns(ncases);
-        for (int i = 0; i < ncases; ++i) {
-            ns[i] = tail_chunks(i, Hb);
-            push_chunks(items, i, nstrip[i], Wi, 0, c.hcases[i].ny - ns[i] * Hs, Hb);
-        }
-        for (int i = 0; i < ncases; ++i)
-            if (ns[i] > 0) push_chunks(items, i, nstrip[i], Wi, c.hcases[i].ny - ns[i] * Hs, c.hcases[i].ny, Hs);
-        c.rows_used = Hb;
     }
     c.nitems = (int)items.size();
+    int Hr = 0;  // all per-case lists resident at once: the height that costs least, if any is
+    double best_r = -1.0;
+    for (int h = 1; h <= 16; ++h) {
+        const double cost = uniform_cost(h);
+        if (cost >= 0 && (best_r < 0 || cost < best_r)) {
+            best_r = cost;
+            Hr = h;
+        }
+    }
     for (int i = 0; i < ncases; ++i) {
         DevCase& d = c.hcases[i];
         // per-case chunk height: minimise (items + resident) x (h + 5) for this case alone
         long long bestc = -1;
-        int Hf = 16;
-        for (int h = 16; h <= 128; ++h) {
+        int Hf = Hr > 0 ? Hr : 16;
+        for (int h = 16; h <= 128 && Hr == 0; ++h) {
             const long long cost = ((long long)nstrip[i] * ((d.ny + h - 1) / h) + resident) * (h + 5);
             if (bestc < 0 || cost < bestc) {
                 bestc = cost;
@@ -326,7 +386,7 @@ lbm_status build_items(Ctx& c) {
             }
         }
         d.item_begin = (int)items.size();
-        push_chunks(items, i, nstrip[i], Wi, 0, d.ny, Hf);
+        push_chunks(items, i, nstrip[i], Wi, 0, d.ny, Hf, Hr == 0);
         d.item_end = (int)items.size();
     }
     c.nitems_all = (int)items.size();
@@ -542,7 +602,10 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
     // work list and launch shape.  Block width: the one that launches fewer thread columns over all
     // cases (windows of width - 8 interior columns; 64 wins on lattices narrower than about 56
     // columns).  The wall-list correction is inlined where wall-list nodes are common (more than 4 %
-    // of the fluid nodes), called out of line otherwise.
+    // of the fluid nodes) or the lattices are large: the call's register saves cost every row
+    // (seven 1024 x 1024 cases, 0.5 % wall-list nodes: 183 us called, 173 inlined; FP16 170 and 150;
+    // 14 of 300 x 350 60.0 and 54.8).  Below about 2^18 nodes a step is a chain of latencies and the two
+    // measure the same.
     {
         long long cols[2] = {0, 0};
         const int widths[2] = {128, 64};
@@ -555,7 +618,7 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
     {
         long long fl = 0;
         for (const HostCase& h : c.cases) fl += h.nfluid;
-        c.wall_inline = (double)c.nwall > 0.04 * (double)fl ? 1 : 0;
+        c.wall_inline = ((double)c.nwall > 0.04 * (double)fl || c.dense_elems > (1LL << 18)) ? 1 : 0;
     }
     st = build_items(c);
     if (st != LBM_OK) return bail(st);
@@ -1125,7 +1188,7 @@ lbm_status lbm_autotune(lbm_ctx* ctx, int32_t steps, double* best_ms) {
     if (steps < 1) return fail(LBM_EINVAL, "steps must be >= 1");
     Ctx& c = ctx->c;
     const int cand_t[] = {128, 64};
-    const int cand_r[] = {0, -8, 16, 32, 64, 128};
+    const int cand_r[] = {0, -8, -16, 16, 32, 64, 128};
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));

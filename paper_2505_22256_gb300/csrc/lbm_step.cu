@@ -974,7 +974,7 @@ __global__ void k_diag_reduce(const DevCase* __restrict__ cases, int c, const do
 template <class S, int T>
 void* kernel_ptr(int variant) {
     using R = typename ComputeOf<S>::type;
-    return variant == 2 ? (void*)k_step<S, R, true, false, T>
+    return variant == 2 ? (void*)k_step<S, R, true, true, T>
                         : (variant == 1 ? (void*)k_step<S, R, false, true, T> : (void*)k_step<S, R, false, false, T>);
 }
 
@@ -1027,7 +1027,7 @@ template <class S, int T>
 cudaError_t launch_step_w(const Ctx& c, const StepArgs& a, cudaStream_t s, bool fields, int grid) {
     using R = typename ComputeOf<S>::type;
     const PdlLaunch l(dim3((unsigned)grid), dim3(T), smem_for<S>(T), s);
-    if (fields) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, true, false, T>, a);
+    if (fields) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, true, true, T>, a);
     if (c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, false, true, T>, a);
     return cudaLaunchKernelEx(&l.cfg, k_step<S, R, false, false, T>, a);
 }
