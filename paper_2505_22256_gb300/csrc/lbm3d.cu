@@ -181,6 +181,8 @@ template <class S, class R>
 __global__ void __launch_bounds__(128) k3_rho(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags,
                                               const Pair<S>* __restrict__ fs, typename Rho2<R>::T* __restrict__ rho) {
     const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
+    pdl_wait();
+    pdl_launch_next();
     if (x >= g.nx || y >= g.ny) return;
     const int s = (z * g.ny + y) * g.nx + x;
     const uint32_t fl = flags[s];
@@ -218,6 +220,44 @@ __device__ __forceinline__ double d3_combine(int q, double a, double b) {
 __device__ __forceinline__ double d3_neutral(int q) {
     return (q == 6 || q == 8) ? INFINITY : (q == 7 || q == 9) ? -INFINITY : 0.0;
 }
+
+// One thread's diagnostics.  The sums are FP64; the extrema compare in the compute type (exact), and
+// |u|^2, taken in FP64, only where its value in the compute type could raise the maximum: FP64
+// operations run at two per SM and cycle, and the record's were what the diagnostics pass waited for.
+template <class R>
+struct Diag3 {
+    double mA = 0.0, mB = 0.0, px = 0.0, py = 0.0, pz = 0.0, u2 = 0.0;
+    R near_u2 = (R)0, aMin = (R)INFINITY, aMax = (R)-INFINITY, bMin = (R)INFINITY, bMax = (R)-INFINITY;
+    int n = 0;
+    bool bad = false;
+    __device__ __forceinline__ void add(R rA, R rB, const R (&u)[3]) {
+        const double dr = (double)(rA + rB);
+        mA += (double)rA;
+        mB += (double)rB;
+        px += dr * (double)u[0];
+        py += dr * (double)u[1];
+        pz += dr * (double)u[2];
+        const R v = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+        // v is within a few roundings of |u|^2 (a denormal or overflowing v says nothing)
+        if (v >= near_u2 * (R)0.9999 || v < (R)1e-30 || !isfinite(v)) {
+            const double w = (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2];
+            u2 = fmax(u2, w);
+            near_u2 = fmax(near_u2, isfinite(v) ? v : (R)0);
+            if (!isfinite(w)) bad = true;
+        }
+        aMin = fmin(aMin, rA);
+        aMax = fmax(aMax, rA);
+        bMin = fmin(bMin, rB);
+        bMax = fmax(bMax, rB);
+        ++n;
+        if (!(rA > (R)0) || !(rB > (R)0) || !isfinite(rA) || !isfinite(rB)) bad = true;
+    }
+    __device__ __forceinline__ void to_record(double (&v)[k3DiagN]) const {
+        v[0] = mA; v[1] = mB; v[2] = px; v[3] = py; v[4] = pz; v[5] = u2;
+        v[6] = (double)aMin; v[7] = (double)aMax; v[8] = (double)bMin; v[9] = (double)bMax;
+        v[10] = (double)n; v[11] = bad ? 1.0 : 0.0;
+    }
+};
 
 // ------------------------------------------------------------------------------------------------
 // Step kernel of the 3-D form.  A block of 32 x 4 columns (x, y) marches over a chunk of z planes.
@@ -297,15 +337,21 @@ __device__ __forceinline__ void wall_stencil3(const V2<R>* b0, const V2<R>* b1, 
 #ifndef LBM3_MIN_BLOCKS
 #define LBM3_MIN_BLOCKS 3
 #endif
-// kFields: the fields form.  In place of the collision each node writes rho_A, rho_B and u (FP64, o5
-// may be NULL) and adds its values to the thread's diagnostic record; each block writes one record
-// (block index blockIdx.x + gridDim.x (blockIdx.y + gridDim.y blockIdx.z)) to part.
-template <class S, class R, int kAdh, bool kFields = false>
+// kMode: kStep collides.  The fields forms write rho_A, rho_B and u (FP64, each of o5 may be NULL) in
+// place of the collision; kFieldsDiag also adds each node's values to the thread's diagnostic record,
+// and each block writes one record (block index blockIdx.x + gridDim.x (blockIdx.y + gridDim.y
+// blockIdx.z)) to part.  Apart, since the FP64 sums of the records run at two operations per SM and
+// cycle: reading the fields of 200 x 200 x 280 took 1.0 ms with them.
+enum { kStep = 0, kFieldsOnly = 1, kFieldsDiag = 2 };
+struct Out5 {
+    double* p[5];
+};
+template <class S, class R, int kAdh, int kMode = kStep>
 __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
     k3_march(Geo3 g, P3<R> P, int zc, const uint32_t* __restrict__ flags, const Pair<S>* __restrict__ fs,
-             const V2<R>* __restrict__ rho, Pair<S>* __restrict__ fout, double* __restrict__ o5,
-             double* __restrict__ part) {
+             const V2<R>* __restrict__ rho, Pair<S>* __restrict__ fout, Out5 o5, double* __restrict__ part) {
     using V = V2<R>;
+    constexpr bool kFields = kMode != kStep, kDiag = kMode == kFieldsDiag;
     extern __shared__ __align__(16) unsigned char smem3[];
     V* ring = reinterpret_cast<V*>(smem3);
     const int tx = threadIdx.x, ty = threadIdx.y, t = ty * k3TX + tx;
@@ -357,11 +403,9 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
         }
     };
 
-    double rec[k3DiagN];  // fields form: this thread's diagnostic record
-    if constexpr (kFields) {
-#pragma unroll
-        for (int q = 0; q < k3DiagN; ++q) rec[q] = d3_neutral(q);
-    }
+    Diag3<R> diag;  // kFieldsDiag
+    pdl_wait();
+    pdl_launch_next();
 
     // prologue: planes z0-2 .. z0+2 into the ring, plane z0+3 into registers, populations of z0
     uint32_t fl_nx = active ? flags[z0 * nxy + yx] : k3Solid;
@@ -454,23 +498,12 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
                 u[d] = ((mv[d].x + mv[d].y) + (R)0.5 * (FA + FB)) * inv;
             }
             if constexpr (kFields) {
-                if (o5) {
-                    o5[s] = (double)rA;
-                    o5[g.N + s] = (double)rB;
-                    o5[2 * g.N + s] = (double)u[0];
-                    o5[3 * g.N + s] = (double)u[1];
-                    o5[4 * g.N + s] = (double)u[2];
-                }
-                const double dr = (double)(rA + rB);
-                // |u|^2; the square root is taken once, of the maximum (it is monotonic)
-                const double u2 = (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2];
-                const bool bad = !(rA > (R)0) || !(rB > (R)0) || !isfinite(u2) || !isfinite((double)rA) ||
-                                 !isfinite((double)rB);
-                const double v[k3DiagN] = {(double)rA,       (double)rB, dr * (double)u[0], dr * (double)u[1],
-                                           dr * (double)u[2], u2,         (double)rA,        (double)rA,
-                                           (double)rB,        (double)rB, 1.0,               bad ? 1.0 : 0.0};
+                if (o5.p[0]) o5.p[0][s] = (double)rA;
+                if (o5.p[1]) o5.p[1][s] = (double)rB;
 #pragma unroll
-                for (int q = 0; q < k3DiagN; ++q) rec[q] = d3_combine(q, rec[q], v[q]);
+                for (int d = 0; d < 3; ++d)
+                    if (o5.p[2 + d]) o5.p[2 + d][s] = (double)u[d];
+                if constexpr (kDiag) diag.add(rA, rB, u);
             } else {
                 // SRT collision with Guo forcing, per pair of directions (e, -e), both components at
                 // once.  With a = e.u, b = e.F_k, P = om rho a + cF b, C0 = om rho (1 - 1.5u^2) - 3 cF u.F:
@@ -513,17 +546,21 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
                 for (int i = 0; i < 19; ++i) st3<S, R>(fout + (long long)i * g.N + s, o[i], P, i);
             }
         } else if constexpr (kFields) {  // solid node: zero fields
-            if (active && o5)
-                for (int q = 0; q < 5; ++q) o5[(long long)q * g.N + s] = 0.0;
+            if (active)
+#pragma unroll
+                for (int q = 0; q < 5; ++q)
+                    if (o5.p[q]) o5.p[q][s] = 0.0;
         }
         if (z + 3 <= z1 + 1) store_plane(z + 3, nxt);
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < k3HN; ++k) nxt[k] = nn[k];
     }
-    if constexpr (kFields) {  // the block's record: warps by shuffles, then the warps in order
+    if constexpr (kDiag) {  // the block's record: warps by shuffles, then the warps in order
         __shared__ double red[k3T / 32][k3DiagN];
         const int lane = t & 31, warp = t >> 5;
+        double rec[k3DiagN];
+        diag.to_record(rec);
 #pragma unroll
         for (int q = 0; q < k3DiagN; ++q) {
             double v = rec[q];
@@ -574,15 +611,14 @@ __global__ void __launch_bounds__(k3DiagMidThreads) k3_diag_mid(long long nblock
     }
 }
 
-// Combine records in record order (one warp; deterministic); max |u| from max |u|^2.
-__global__ void k3_diag_final(long long nblocks, const double* __restrict__ part, double* __restrict__ out) {
-    const int lane = threadIdx.x;
-    for (int q = 0; q < k3DiagN; ++q) {
-        double v = d3_neutral(q);
-        for (long long b = lane; b < nblocks; b += 32) v = d3_combine(q, v, part[b * k3DiagN + q]);
-        for (int off = 16; off > 0; off >>= 1) v = d3_combine(q, v, __shfl_xor_sync(0xffffffffu, v, off));
-        if (lane == 0) out[q] = q == 5 ? sqrt(v) : v;
-    }
+// Combine records in record order (one warp per value; deterministic); max |u| from max |u|^2.
+__global__ void __launch_bounds__(32 * k3DiagN) k3_diag_final(long long nblocks, const double* __restrict__ part,
+                                                             double* __restrict__ out) {
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double v = d3_neutral(q);
+    for (long long b = lane; b < nblocks; b += 32) v = d3_combine(q, v, part[b * k3DiagN + q]);
+    for (int off = 16; off > 0; off >>= 1) v = d3_combine(q, v, __shfl_xor_sync(0xffffffffu, v, off));
+    if (lane == 0) out[q] = q == 5 ? sqrt(v) : v;
 }
 
 // post-streaming populations (FP64 [2][19][N]) <-> post-collision buffer
@@ -711,8 +747,10 @@ __global__ void __launch_bounds__(kR3T) k3_set_rest(Geo3 g, P3<R> P, const uint3
 // Contact angle on a sphere (FP64): interface points, algebraic sphere fit, one Gauss-Newton step
 // ------------------------------------------------------------------------------------------------
 constexpr int kC3Threads = 256;
-constexpr int kC3Blocks = 608;  // fixed (the summation order does not depend on the device): 4 x 152
+constexpr int kC3Blocks = 304;  // fixed: the summation order does not depend on the device
 constexpr int kC3Vals = 14;
+constexpr int kC3Seg = 4 * kC3Threads;  // nodes of a block of k3_ca_cross
+constexpr int kC3Group = 4 * kC3Seg;    // nodes a block of a pass works on together
 
 template <class R>
 struct Ca3 {
@@ -720,13 +758,13 @@ struct Ca3 {
     const uint32_t* flags;
     const typename Rho2<R>::T* rho;  // interleaved (rho_A, rho_B)
     uint8_t* cross;                  // per node: bit a set where the link to the +a neighbour crosses
-};                                   // rho^e = 0 (written by pass 0, read by the later passes)
-
-template <class R>
-__device__ __forceinline__ bool ca3_usable(const Ca3<R>& c, long long s) { return (c.flags[s] & (k3Solid | k3Near)) == 0; }
+                                     // rho^e = 0 (written by k3_ca_cross, read by the passes)
+    int* count;                      // links that cross, per kC3Seg nodes
+};
 
 __device__ __forceinline__ double phi3(double a, double b) { return (a - b) / (a + b); }
 __device__ __forceinline__ bool phi3_pos(double a, double b) {
+    if (a == b) return false;  // 0 or undefined; solid sites hold equal values, and take no division
     const double sum = a + b;
     return (sum > 0.0 && sum < INFINITY) ? a > b : phi3(a, b) > 0.0;
 }
@@ -735,109 +773,161 @@ __device__ __forceinline__ bool phi3_pos(double a, double b) {
 // sum; the comparison is exact in either type), so FP32 takes it without the FP64 pipe; every other
 // case goes through the FP64 form.  The decision is the FP64 one bit for bit.
 __device__ __forceinline__ bool phi3_pos_r(float a, float b) {
+    if (a == b) return false;
     if (isfinite(a) && isfinite(b) && a + b > 0.0f) return a > b;
     return phi3_pos((double)a, (double)b);
 }
 __device__ __forceinline__ bool phi3_pos_r(double a, double b) { return phi3_pos(a, b); }
 
 // st: 0 N, 1-3 centroid, 4-6 centre, 7 r, 8 rms, 9 theta, 10 status (1: too few points)
-// One kernel per pass (kPass 0: count and centroid, 1: algebraic fit sums, 2: Gauss-Newton sums, 3:
-// residual), so that each holds only the sums it needs: the pass is bound by the latency of its
-// dependent loads, and fewer registers keep more warps resident.
+// Crossing links of every node.  The links of a node are tested by the signs of rho^e alone, a thread's
+// four nodes and their neighbours in flight together; flags and coordinates (a usable pair of nodes, no
+// pair across the periodic seam) are looked at only where a sign changes.  As part of a pass over all
+// nodes that looked at the flags first, one node after the other, it took 387 us on 200 x 200 x 280.
+template <class R>
+__global__ void __launch_bounds__(kC3Threads) k3_ca_cross(Ca3<R> c) {
+    const unsigned nx = c.g.nx, ny = c.g.ny, n = (unsigned)c.g.N;  // N < 2^31
+    const unsigned base = blockIdx.x * kC3Seg + threadIdx.x;
+    const unsigned step[3] = {1u, nx, nx * ny};
+    typename Rho2<R>::T r[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const unsigned s = min(base + j * kC3Threads, n - 1);
+        r[j][0] = c.rho[s];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) r[j][1 + a] = c.rho[min(s + step[a], n - 1)];
+    }
+    uint32_t change[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const bool p = phi3_pos_r(r[j][0].x, r[j][0].y);
+        change[j] = 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            if (p != phi3_pos_r(r[j][1 + a].x, r[j][1 + a].y)) change[j] |= 1u << a;
+        if (base + j * kC3Threads >= n) change[j] = 0;
+    }
+    int links = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const unsigned s = base + j * kC3Threads;
+        uint32_t found = 0;
+        if (change[j]) {
+            const unsigned row = s / nx, at[3] = {s - row * nx, row % ny, row / ny};
+            const unsigned lim[3] = {nx, ny, (unsigned)c.g.nz};
+            uint32_t fl[4];
+            fl[0] = c.flags[s];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) fl[1 + a] = c.flags[min(s + step[a], n - 1)];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                if ((change[j] >> a & 1u) && at[a] + 1 < lim[a] && ((fl[0] | fl[1 + a]) & (k3Solid | k3Near)) == 0)
+                    found |= 1u << a;
+        }
+        c.cross[s] = (uint8_t)found;  // the array is padded to whole groups
+        links += __popc(found);
+    }
+    __shared__ int red[kC3Threads / 32];
+    links = __reduce_add_sync(0xffffffffu, links);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = links;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int v = 0;
+        for (int w = 0; w < kC3Threads / 32; ++w) v += red[w];
+        c.count[blockIdx.x] = v;
+    }
+}
+
+// st: 0 N, 1-3 centroid, 4-6 centre, 7 r, 8 rms, 9 theta, 10 status (1: too few points)
+// One kernel per pass over the crossing links (kPass 0: count and centroid, 1: algebraic fit sums, 2:
+// Gauss-Newton sums, 3: residual), so that each holds only the sums it needs.  Block b takes the
+// groups of nodes b, b + gridDim.x, ... that hold any link (most hold none) and packs a group's links in
+// node order, so that whole warps work on them: the FP64 divisions of a link cost a warp as much as
+// those of 32.
 template <class R, int kPass>
-__global__ void __launch_bounds__(kC3Threads) k3_ca_pass(Ca3<R> c, const double* __restrict__ st,
+__global__ void __launch_bounds__(kC3Threads) k3_ca_pass(Ca3<R> c, int ngroup, const double* __restrict__ st,
                                                         double* __restrict__ part) {
     constexpr int pass = kPass;
     constexpr int nv = pass == 0 ? 4 : pass == 1 ? 13 : pass == 2 ? 14 : 1;  // sums this pass forms
+    __shared__ uint16_t keys[3 * kC3Group];  // 4 x node within the group + axis
+    __shared__ int warp_sum[kC3Threads / 32];
     double acc[kC3Vals];
 #pragma unroll
     for (int q = 0; q < kC3Vals; ++q) acc[q] = 0.0;
     const double m0 = st[1], m1 = st[2], m2 = st[3], c0 = st[4], c1 = st[5], c2 = st[6], r = st[7];
-    const Geo3& g = c.g;
-    const bool small = g.N < (1LL << 31);  // node index and coordinates in 32-bit arithmetic
-    // one node: pass 0 tests its three links and records the crossings, the later passes take the
-    // recorded ones (bits)
-    auto node = [&](long long s, uint32_t bits) {
-        int x, y, z;
-        if (small) {
-            const unsigned su = (unsigned)s, row = su / (unsigned)g.nx;
-            x = (int)(su - row * (unsigned)g.nx);
-            z = (int)(row / (unsigned)g.ny);
-            y = (int)(row - (unsigned)z * (unsigned)g.ny);
+    const unsigned nx = c.g.nx, ny = c.g.ny;
+    auto link = [&](unsigned s, int axis) {
+        const unsigned row = s / nx;
+        const typename Rho2<R>::T r0 = c.rho[s], r1 = c.rho[s + (axis == 0 ? 1u : (axis == 1 ? nx : nx * ny))];
+        const double a = phi3((double)r0.x, (double)r0.y), b = phi3((double)r1.x, (double)r1.y), d = a / (a - b);
+        const double p[3] = {(double)(s - row * nx) + (axis == 0 ? d : 0.0), (double)(row % ny) + (axis == 1 ? d : 0.0),
+                             (double)(row / ny) + (axis == 2 ? d : 0.0)};
+        if constexpr (pass == 0) {
+            acc[0] += 1.0;
+            acc[1] += p[0];
+            acc[2] += p[1];
+            acc[3] += p[2];
+        } else if constexpr (pass == 1) {
+            const double q0 = p[0] - m0, q1 = p[1] - m1, q2 = p[2] - m2, qq = q0 * q0 + q1 * q1 + q2 * q2;
+            acc[0] += q0 * q0; acc[1] += q0 * q1; acc[2] += q0 * q2;
+            acc[3] += q1 * q1; acc[4] += q1 * q2; acc[5] += q2 * q2;
+            acc[6] += q0; acc[7] += q1; acc[8] += q2;
+            acc[9] += q0 * qq; acc[10] += q1 * qq; acc[11] += q2 * qq; acc[12] += qq;
+        } else if constexpr (pass == 2) {
+            const double d0 = p[0] - c0, d1 = p[1] - c1, d2 = p[2] - c2;
+            const double dd = sqrt(d0 * d0 + d1 * d1 + d2 * d2), res = dd - r;
+            const double j[4] = {-d0 / dd, -d1 / dd, -d2 / dd, -1.0};
+            int k = 0;
+#pragma unroll
+            for (int a2 = 0; a2 < 4; ++a2)
+#pragma unroll
+                for (int b2 = a2; b2 < 4; ++b2) acc[k++] += j[a2] * j[b2];
+#pragma unroll
+            for (int a2 = 0; a2 < 4; ++a2) acc[10 + a2] += j[a2] * res;
         } else {
-            x = (int)(s % g.nx);
-            y = (int)((s / g.nx) % g.ny);
-            z = (int)(s / ((long long)g.nx * g.ny));
+            const double d0 = p[0] - c0, d1 = p[1] - c1, d2 = p[2] - c2;
+            const double res = sqrt(d0 * d0 + d1 * d1 + d2 * d2) - r;
+            acc[0] += res * res;
         }
-        const typename Rho2<R>::T r0 = c.rho[s];
-        const double ra = (double)r0.x, rb = (double)r0.y;
-        const bool pa = phi3_pos_r(r0.x, r0.y);
-        uint32_t found = 0;
-        for (int axis = 0; axis < 3; ++axis) {
-            const long long sn = s + (axis == 0 ? 1 : (axis == 1 ? (long long)g.nx : (long long)g.nx * g.ny));
-            if constexpr (pass == 0) {
-                const int lim = axis == 0 ? g.nx : (axis == 1 ? g.ny : g.nz);
-                const int coord = axis == 0 ? x : (axis == 1 ? y : z);
-                if (coord + 1 >= lim) continue;  // no pair across the periodic seam
-                if (!ca3_usable(c, sn)) continue;
-                const typename Rho2<R>::T r1 = c.rho[sn];
-                if (pa == phi3_pos_r(r1.x, r1.y)) continue;
-                found |= 1u << axis;
-            } else if (!((bits >> axis) & 1u)) {
-                continue;
-            }
-            const typename Rho2<R>::T r1 = c.rho[sn];
-            const double qa = (double)r1.x, qb = (double)r1.y;
-            const double a = phi3(ra, rb), b = phi3(qa, qb);
-            double p[3] = {(double)x, (double)y, (double)z};
-            p[axis] += a / (a - b);
-            if constexpr (pass == 0) {
-                acc[0] += 1.0;
-                acc[1] += p[0];
-                acc[2] += p[1];
-                acc[3] += p[2];
-            } else if constexpr (pass == 1) {
-                const double q0 = p[0] - m0, q1 = p[1] - m1, q2 = p[2] - m2, qq = q0 * q0 + q1 * q1 + q2 * q2;
-                acc[0] += q0 * q0; acc[1] += q0 * q1; acc[2] += q0 * q2;
-                acc[3] += q1 * q1; acc[4] += q1 * q2; acc[5] += q2 * q2;
-                acc[6] += q0; acc[7] += q1; acc[8] += q2;
-                acc[9] += q0 * qq; acc[10] += q1 * qq; acc[11] += q2 * qq; acc[12] += qq;
-            } else if constexpr (pass == 2) {
-                const double d0 = p[0] - c0, d1 = p[1] - c1, d2 = p[2] - c2;
-                const double d = sqrt(d0 * d0 + d1 * d1 + d2 * d2), res = d - r;
-                const double j[4] = {-d0 / d, -d1 / d, -d2 / d, -1.0};
-                int k = 0;
-                for (int a2 = 0; a2 < 4; ++a2)
-                    for (int b2 = a2; b2 < 4; ++b2) acc[k++] += j[a2] * j[b2];
-                for (int a2 = 0; a2 < 4; ++a2) acc[10 + a2] += j[a2] * res;
-            } else {
-                const double d0 = p[0] - c0, d1 = p[1] - c1, d2 = p[2] - c2;
-                const double res = sqrt(d0 * d0 + d1 * d1 + d2 * d2) - r;
-                acc[0] += res * res;
-            }
-        }
-        if constexpr (pass == 0) c.cross[s] = (uint8_t)found;
     };
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
-    // one node per thread and step, so that the crossings of neighbouring nodes (they cluster along
-    // the interface) go to neighbouring lanes
-    if constexpr (pass == 0) {
-        for (long long s = tid; s < g.N; s += nth) {
-            if (ca3_usable(c, s)) node(s, 0u);
-            else c.cross[s] = 0;
-        }
-    } else {  // the same order; the bits of four steps are loaded together
-        for (long long s0 = tid; s0 < g.N; s0 += 4 * nth) {
-            uint32_t b[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = (int)gridDim.x;
+    for (int first = blockIdx.x; first < ngroup; first += 32 * nb) {  // the counts of 32 groups together
+        const long long mine = (long long)first + (long long)lane * nb;
+        int4 n4 = make_int4(0, 0, 0, 0);
+        if (mine < ngroup) n4 = reinterpret_cast<const int4*>(c.count)[mine];
+        uint32_t left = __ballot_sync(0xffffffffu, (n4.x | n4.y | n4.z | n4.w) != 0);
+        while (left) {  // the same in every warp
+            const unsigned group = (unsigned)first + (unsigned)(__ffs(left) - 1) * nb;
+            left &= left - 1;
+            const uint4 w = *reinterpret_cast<const uint4*>(c.cross + (size_t)group * kC3Group + 16 * threadIdx.x);
+            const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+            const int mylinks = __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+            int at = mylinks;  // inclusive prefix over the block's threads
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = s0 + j * nth < g.N ? c.cross[s0 + j * nth] : 0u;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, at, off);
+                if (lane >= off) at += o;
+            }
+            if (lane == 31) warp_sum[warp] = at;
+            __syncthreads();
+            int total = 0;
+            for (int k = 0; k < kC3Threads / 32; ++k) {
+                if (k < warp) at += warp_sum[k];
+                total += warp_sum[k];
+            }
+            at -= mylinks;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (b[j]) node(s0 + j * nth, b[j]);
+            for (int k = 0; k < 4; ++k)
+                for (uint32_t v = ws[k]; v; v &= v - 1) {  // bit 8 node + axis
+                    const int b = __ffs(v) - 1;
+                    keys[at++] = (uint16_t)((16 * threadIdx.x + 4 * k + (b >> 3)) * 4 + (b & 7));
+                }
+            __syncthreads();
+            for (int k = threadIdx.x; k < total; k += kC3Threads) link(group * kC3Group + (keys[k] >> 2), keys[k] & 3);
+            __syncthreads();
         }
     }
     __shared__ double red[kC3Threads / 32][kC3Vals];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < nv; ++q) {
         double v = acc[q];
@@ -845,13 +935,12 @@ __global__ void __launch_bounds__(kC3Threads) k3_ca_pass(Ca3<R> c, const double*
         if (lane == 0) red[warp][q] = v;
     }
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int q = 0; q < kC3Vals; ++q) {  // the sums a pass does not form are written as 0
-            double v = 0.0;
-            if (q < nv)
-                for (int w = 0; w < kC3Threads / 32; ++w) v += red[w][q];
-            part[blockIdx.x * kC3Vals + q] = v;
-        }
+    if (threadIdx.x < kC3Vals) {  // the sums a pass does not form are written as 0
+        double v = 0.0;
+        if ((int)threadIdx.x < nv)
+            for (int w = 0; w < kC3Threads / 32; ++w) v += red[w][threadIdx.x];
+        part[blockIdx.x * kC3Vals + threadIdx.x] = v;
+    }
 }
 
 __device__ void solve4(double A[4][4], double b[4], double x[4]) {
@@ -880,17 +969,17 @@ __device__ void solve4(double A[4][4], double b[4], double x[4]) {
     }
 }
 
-__global__ void k3_ca_solve(int pass, int nblocks, const double* __restrict__ part, double* __restrict__ st, double sc0,
-                            double sc1, double sc2, double R) {
-    double S[kC3Vals];
-    const int lane = threadIdx.x & 31;
-    for (int q = 0; q < kC3Vals; ++q) {
-        double v = 0.0;
-        for (int b = lane; b < nblocks; b += 32) v += part[b * kC3Vals + q];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        S[q] = v;
-    }
-    if (lane != 0) return;
+__global__ void __launch_bounds__(32 * kC3Vals) k3_ca_solve(int pass, int nblocks, const double* __restrict__ part,
+                                                           double* __restrict__ st, double sc0, double sc1, double sc2,
+                                                           double R) {
+    __shared__ double S[kC3Vals];  // one warp per sum
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double v = 0.0;
+    for (int b = lane; b < nblocks; b += 32) v += part[b * kC3Vals + q];
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (lane == 0) S[q] = v;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     if (pass == 0) {
         st[0] = S[0];
         st[10] = S[0] < 8.0 ? 1.0 : 0.0;
@@ -951,12 +1040,14 @@ struct lbm3d_ctx {
     uint32_t* flags = nullptr;
     unsigned char* f[2] = {nullptr, nullptr};
     int cur = 0;
-    unsigned char* rho = nullptr;  // [2][N] in the compute type
+    unsigned char* rho = nullptr;  // [N] density pairs in the compute type
+    int zc = 0;                    // z planes per block of the march
     double* part = nullptr;        // per-block diagnostic records
     long long nparts = 0;
     double* dout = nullptr;        // [k3DiagN]
     double* ca = nullptr;          // contact angle: status record + block partials
-    uint8_t* ca_cross = nullptr;   // contact angle: per-node crossing bits (N bytes)
+    uint8_t* ca_cross = nullptr;   // contact angle: per-node crossing bits (N bytes, whole groups)
+    int* ca_count = nullptr;       // crossings per kC3Seg nodes
     double* scratch = nullptr;     // [38][N] doubles for population transfers and fields (on demand)
     double* dens = nullptr;        // [2][N] doubles for lbm3d_set_densities from host arrays (on demand)
     // overlapped host transfers (lbm3d_set_densities_async, lbm3d_fields_async; on first use): copy
@@ -1018,13 +1109,29 @@ cudaError_t with_types3(int storage, Fn&& fn) {
 dim3 grid3(const Geo3& g) { return dim3((unsigned)((g.nx + 31) / 32), (unsigned)((g.ny + 3) / 4), (unsigned)g.nz); }
 const dim3 kBlock3(32, 4, 1);
 
-// z planes per block of the step kernel: about 16, spread evenly over nz
+// z planes per block of the march.  A block costs its planes plus about 2 (the first density planes, the
+// start), and a launch runs its blocks in rounds of `resident`; about 16 planes, spread evenly over
+// nz, once there are many rounds (32 measured the same).  With 16 planes for every lattice a small
+// one ran as a few blocks: 40 x 40 x 56, 80 blocks, 39 us a step; with this rule 18.
 #ifndef LBM3_ZCHUNK
 #define LBM3_ZCHUNK 16
 #endif
-int zchunk3(const Geo3& g) {
-    const int chunks = (g.nz + LBM3_ZCHUNK - 1) / LBM3_ZCHUNK;
-    return (g.nz + chunks - 1) / chunks;
+int zchunk3(const Geo3& g, int resident) {
+    const long long tiles = (long long)((g.nx + k3TX - 1) / k3TX) * ((g.ny + k3TY - 1) / k3TY);
+    double best = -1.0;
+    int zc = LBM3_ZCHUNK;
+    for (int n = (g.nz + LBM3_ZCHUNK - 1) / LBM3_ZCHUNK; n <= g.nz; ++n) {
+        const int h = (g.nz + n - 1) / n;
+        const long long blocks = tiles * ((g.nz + h - 1) / h);
+        const double rounds = blocks > 3LL * resident ? (double)blocks / resident + 0.5
+                                                      : (double)((blocks + resident - 1) / resident);
+        const double cost = rounds * (h + 2);
+        if (best < 0 || cost < best) {
+            best = cost;
+            zc = h;
+        }
+    }
+    return zc;
 }
 
 cudaError_t scratch_for(lbm3d_ctx* c) {
@@ -1042,54 +1149,61 @@ Pair<S>* state3(const lbm3d_ctx* c, int buf) {
     return reinterpret_cast<Pair<S>*>(c->f[buf]);
 }
 
-// the step kernel instance of the adhesion variant (kFields: its fields form)
-template <class S, class R, bool kFields = false>
+// the march kernel instance of the adhesion variant
+template <class S, class R, int kMode = kStep>
 auto march_kernel(const P3<R>& P) {
-    return P.adh ? k3_march<S, R, kAdhD3Q19, kFields>
-                 : (P.psi ? k3_march<S, R, kAdhE8Psi, kFields> : k3_march<S, R, kAdhE8, kFields>);
+    return P.adh ? k3_march<S, R, kAdhD3Q19, kMode>
+                 : (P.psi ? k3_march<S, R, kAdhE8Psi, kMode> : k3_march<S, R, kAdhE8, kMode>);
 }
 
 dim3 march_grid(const Geo3& g, int zc) {
     return dim3((unsigned)((g.nx + k3TX - 1) / k3TX), (unsigned)((g.ny + k3TY - 1) / k3TY), (unsigned)((g.nz + zc - 1) / zc));
 }
 
+// densities of the current state into c->rho
 template <class S, class R>
-cudaError_t step_once(lbm3d_ctx* c) {
-    const dim3 gr = grid3(c->g);
-    const Pair<S>* fs = state3<S>(c, c->cur);
-    auto* rho = reinterpret_cast<typename Rho2<R>::T*>(c->rho);
-    const P3<R>& P = p3_of<R>(c);
-    k3_rho<S, R><<<gr, kBlock3, 0, c->stream>>>(c->g, P, c->flags, fs, rho);
-    const int zc = zchunk3(c->g);
-    auto* kern = march_kernel<S, R>(P);
-    kern<<<march_grid(c->g, zc), kBlock3, k3_march_smem<R>(), c->stream>>>(
-        c->g, P, zc, c->flags, fs, reinterpret_cast<const V2<R>*>(rho), state3<S>(c, 1 - c->cur), nullptr, nullptr);
-    c->cur ^= 1;
-    return cudaGetLastError();
+cudaError_t launch_rho3(lbm3d_ctx* c) {
+    const PdlLaunch l(grid3(c->g), kBlock3, 0, c->stream);
+    return cudaLaunchKernelEx(&l.cfg, k3_rho<S, R>, c->g, p3_of<R>(c), (const uint32_t*)c->flags,
+                              (const Pair<S>*)state3<S>(c, c->cur), reinterpret_cast<typename Rho2<R>::T*>(c->rho));
 }
 
-// densities of the current state into c->rho, then the fields form of the step kernel (o5 may be
-// NULL): the same pull, stencil sums, moments and forces as a step, per-block diagnostic records
-cudaError_t run_fields(lbm3d_ctx* c, double* o5, bool diag) {
+// the march over the whole lattice; the density pass comes first
+template <class S, class R, int kMode>
+cudaError_t launch_march3(lbm3d_ctx* c, const Out5& o5) {
+    const P3<R>& P = p3_of<R>(c);
+    const PdlLaunch l(march_grid(c->g, c->zc), kBlock3, k3_march_smem<R>(), c->stream);
+    auto* kern = march_kernel<S, R, kMode>(P);
+    if (k3_march_smem<R>() > 48 * 1024) {  // above the default limit (FP64)
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k3_march_smem<R>());
+        if (e != cudaSuccess) return e;
+    }
+    return cudaLaunchKernelEx(&l.cfg, kern, c->g, P, c->zc, (const uint32_t*)c->flags, (const Pair<S>*)state3<S>(c, c->cur),
+                              (const V2<R>*)c->rho, state3<S>(c, 1 - c->cur), o5, c->part);
+}
+
+template <class S, class R>
+cudaError_t step_once(lbm3d_ctx* c) {
+    cudaError_t e = launch_rho3<S, R>(c);
+    if (e == cudaSuccess) e = launch_march3<S, R, kStep>(c, Out5{});
+    c->cur ^= 1;
+    return e;
+}
+
+// densities of the current state into c->rho, then a fields form of the march (outputs may be NULL):
+// the same pull, stencil sums, moments and forces as a step; diag: per-block diagnostic records,
+// combined into c->dout
+cudaError_t run_fields(lbm3d_ctx* c, const Out5& o5, bool diag) {
     return with_types3(c->storage, [&](auto* s_, auto* r_) {
         TYPES3(s_, r_);
-        const Pair<S>* fs = state3<S>(c, c->cur);
-        auto* rho = reinterpret_cast<typename Rho2<R>::T*>(c->rho);
-        const P3<R>& P = p3_of<R>(c);
-        k3_rho<S, R><<<grid3(c->g), kBlock3, 0, c->stream>>>(c->g, P, c->flags, fs, rho);
-        const int zc = zchunk3(c->g);
-        const dim3 gm = march_grid(c->g, zc);
-        auto* kern = march_kernel<S, R, true>(P);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k3_march_smem<R>());
-        if (e != cudaSuccess) return e;
-        kern<<<gm, kBlock3, k3_march_smem<R>(), c->stream>>>(c->g, P, zc, c->flags, fs, reinterpret_cast<const V2<R>*>(rho),
-                                                             nullptr, o5, c->part);
-        if (diag) {
-            const long long nb = (long long)gm.x * gm.y * gm.z;  // <= c->nparts (one record per block)
-            double* mid = c->part + c->nparts * k3DiagN;         // k3DiagMid records after the per-block ones
-            k3_diag_mid<<<k3DiagMid, k3DiagMidThreads, 0, c->stream>>>(nb, c->part, mid);
-            k3_diag_final<<<1, 32, 0, c->stream>>>(k3DiagMid, mid, c->dout);
-        }
+        cudaError_t e = launch_rho3<S, R>(c);
+        if (e == cudaSuccess) e = diag ? launch_march3<S, R, kFieldsDiag>(c, o5) : launch_march3<S, R, kFieldsOnly>(c, o5);
+        if (e != cudaSuccess || !diag) return e;
+        const dim3 gm = march_grid(c->g, c->zc);
+        const long long nb = (long long)gm.x * gm.y * gm.z;  // <= c->nparts (one record per block)
+        double* mid = c->part + c->nparts * k3DiagN;         // k3DiagMid records after the per-block ones
+        k3_diag_mid<<<k3DiagMid, k3DiagMidThreads, 0, c->stream>>>(nb, c->part, mid);
+        k3_diag_final<<<1, 32 * k3DiagN, 0, c->stream>>>(k3DiagMid, mid, c->dout);
         return cudaGetLastError();
     });
 }
@@ -1097,9 +1211,7 @@ cudaError_t run_fields(lbm3d_ctx* c, double* o5, bool diag) {
 cudaError_t density_pass(lbm3d_ctx* c) {
     return with_types3(c->storage, [&](auto* s_, auto* r_) {
         TYPES3(s_, r_);
-        k3_rho<S, R><<<grid3(c->g), kBlock3, 0, c->stream>>>(c->g, p3_of<R>(c), c->flags, state3<S>(c, c->cur),
-                                                           reinterpret_cast<typename Rho2<R>::T*>(c->rho));
-        return cudaGetLastError();
+        return launch_rho3<S, R>(c);
     });
 }
 
@@ -1123,15 +1235,17 @@ cudaError_t set_rest3(lbm3d_ctx* c, const double* a, const double* b) {
 
 template <class R>
 cudaError_t ca_passes(lbm3d_ctx* c, const double* sc, double R_) {
-    Ca3<R> ca{c->g, c->flags, reinterpret_cast<const typename Rho2<R>::T*>(c->rho), c->ca_cross};
+    const int ngroup = (int)((c->g.N + kC3Group - 1) / kC3Group);
+    Ca3<R> ca{c->g, c->flags, reinterpret_cast<const typename Rho2<R>::T*>(c->rho), c->ca_cross, c->ca_count};
     double* st = c->ca;
     double* part = c->ca + 16;
     cudaError_t e = cudaMemsetAsync(st, 0, 16 * sizeof(double), c->stream);
     if (e != cudaSuccess) return e;
+    k3_ca_cross<R><<<ngroup * (kC3Group / kC3Seg), kC3Threads, 0, c->stream>>>(ca);
     for (int pass = 0; pass < 4; ++pass) {
         auto* kern = pass == 0 ? k3_ca_pass<R, 0> : pass == 1 ? k3_ca_pass<R, 1> : pass == 2 ? k3_ca_pass<R, 2> : k3_ca_pass<R, 3>;
-        kern<<<kC3Blocks, kC3Threads, 0, c->stream>>>(ca, st, part);
-        k3_ca_solve<<<1, 32, 0, c->stream>>>(pass, kC3Blocks, part, st, sc[0], sc[1], sc[2], R_);
+        kern<<<kC3Blocks, kC3Threads, 0, c->stream>>>(ca, ngroup, st, part);
+        k3_ca_solve<<<1, 32 * kC3Vals, 0, c->stream>>>(pass, kC3Blocks, part, st, sc[0], sc[1], sc[2], R_);
     }
     return cudaGetLastError();
 }
@@ -1153,7 +1267,7 @@ void free_xfer3(lbm3d_ctx* c) {
 
 void free3(lbm3d_ctx* c) {
     free_xfer3(c);
-    void* ptrs[] = {c->solid, c->flags, c->f[0], c->f[1], c->rho, c->part, c->dout, c->ca, c->ca_cross, c->scratch, c->dens};
+    void* ptrs[] = {c->solid, c->flags, c->f[0], c->f[1], c->rho, c->part, c->dout, c->ca, c->ca_cross, c->ca_count, c->scratch, c->dens};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
@@ -1241,6 +1355,7 @@ extern "C" lbm_status lbm3d_create(const lbm3d_grid* grid, const uint8_t* solid,
     }
     const dim3 gr = grid3(c->g);
     c->nparts = (long long)gr.x * gr.y * gr.z;
+    c->zc = zchunk3(c->g, (storage == LBM_STORE_F64 ? 2 : LBM3_MIN_BLOCKS) * prop.multiProcessorCount);
     STEP3(cudaMalloc(&c->solid, N), "mask");
     STEP3(cudaMalloc(&c->flags, N * sizeof(uint32_t)), "flags");
     STEP3(cudaMalloc(&c->f[0], 38 * N * c->elem), "population buffer");
@@ -1249,7 +1364,9 @@ extern "C" lbm_status lbm3d_create(const lbm3d_grid* grid, const uint8_t* solid,
     STEP3(cudaMalloc(&c->part, (c->nparts + k3DiagMid) * k3DiagN * sizeof(double)), "diagnostics");
     STEP3(cudaMalloc(&c->dout, k3DiagN * sizeof(double)), "diagnostics");
     STEP3(cudaMalloc(&c->ca, (16 + kC3Blocks * kC3Vals) * sizeof(double)), "contact-angle scratch");
-    STEP3(cudaMalloc(&c->ca_cross, (size_t)c->g.N), "contact-angle scratch");
+    const size_t ngroup = ((size_t)N + kC3Group - 1) / kC3Group;
+    STEP3(cudaMalloc(&c->ca_cross, ngroup * kC3Group), "contact-angle scratch");
+    STEP3(cudaMalloc(&c->ca_count, ngroup * (kC3Group / kC3Seg) * sizeof(int)), "contact-angle scratch");
     STEP3(cudaMemsetAsync(c->f[0], 0, 38 * N * c->elem, c->stream), "memset");
     STEP3(cudaMemsetAsync(c->f[1], 0, 38 * N * c->elem, c->stream), "memset");
     STEP3(cudaMemcpy(c->solid, solid, N, cudaMemcpyHostToDevice), "mask upload");
@@ -1281,10 +1398,7 @@ extern "C" lbm_status lbm3d_step(lbm3d_ctx* c, int64_t n) {
     TRY3(with_types3(c->storage,
                      [&](auto* s_, auto* r_) {
                          TYPES3(s_, r_);
-                         // the step kernel's shared-memory ring exceeds the default dynamic limit in FP64
-                         cudaError_t e = cudaFuncSetAttribute(march_kernel<S, R>(p3_of<R>(c)),
-                                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                              (int)k3_march_smem<R>());
+                         cudaError_t e = cudaSuccess;
                          for (int64_t t = 0; t < n && e == cudaSuccess; ++t) e = step_once<S, R>(c);
                          return e;
                      }),
@@ -1296,16 +1410,20 @@ extern "C" lbm_status lbm3d_fields(lbm3d_ctx* c, double* rA, double* rB, double*
                                    int32_t on_device) {
     NvtxRange nvtx_("lbm3d_fields");
     if (!c) return report_error(LBM_EINVAL, "NULL context");
+    Out5 outs{{rA, rB, ux, uy, uz}};
+    if (on_device) {
+        TRY3(run_fields(c, outs, false), "fields kernels");
+        return LBM_OK;
+    }
     TRY3(scratch_for(c), "fields scratch");
-    TRY3(run_fields(c, c->scratch, false), "fields kernels");
-    double* outs[5] = {rA, rB, ux, uy, uz};
     const long long N = c->g.N;
+    Out5 dev;
+    for (int q = 0; q < 5; ++q) dev.p[q] = outs.p[q] ? c->scratch + q * N : nullptr;
+    TRY3(run_fields(c, dev, false), "fields kernels");
     for (int q = 0; q < 5; ++q)
-        if (outs[q])
-            TRY3(cudaMemcpyAsync(outs[q], c->scratch + q * N, N * sizeof(double),
-                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream),
-                 "fields copy");
-    if (!on_device) TRY3(cudaStreamSynchronize(c->stream), "fields");
+        if (outs.p[q])
+            TRY3(cudaMemcpyAsync(outs.p[q], dev.p[q], N * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "fields copy");
+    TRY3(cudaStreamSynchronize(c->stream), "fields");
     return LBM_OK;
 }
 
@@ -1367,10 +1485,12 @@ extern "C" lbm_status lbm3d_fields_async(lbm3d_ctx* c, double* rho_A, double* rh
     // the fields pass may overwrite this staging buffer once its previous copy to the host is done;
     // the copies then run on their own stream, beside the context's next work
     TRY3(cudaStreamWaitEvent(c->stream, c->xout_free[k], 0), "transfer order");
-    TRY3(run_fields(c, c->xout[k], false), "fields kernels");
+    double* outs[5] = {rho_A, rho_B, ux, uy, uz};
+    Out5 dev;
+    for (int q = 0; q < 5; ++q) dev.p[q] = outs[q] ? c->xout[k] + q * N : nullptr;
+    TRY3(run_fields(c, dev, false), "fields kernels");
     TRY3(cudaEventRecord(c->xout_ready[k], c->stream), "transfer order");
     TRY3(cudaStreamWaitEvent(c->xs_out, c->xout_ready[k], 0), "transfer order");
-    double* outs[5] = {rho_A, rho_B, ux, uy, uz};
     for (int q = 0; q < 5; ++q)
         if (outs[q])
             TRY3(cudaMemcpyAsync(outs[q], c->xout[k] + q * N, N * sizeof(double), cudaMemcpyDeviceToHost, c->xs_out),
@@ -1432,7 +1552,7 @@ extern "C" lbm_status lbm3d_set_populations(lbm3d_ctx* c, const double* f) {
 
 extern "C" lbm_status lbm3d_diagnostics(lbm3d_ctx* c, lbm3d_diag* out) {
     if (!c || !out) return report_error(LBM_EINVAL, "NULL argument");
-    TRY3(run_fields(c, nullptr, true), "diagnostics kernels");
+    TRY3(run_fields(c, Out5{}, true), "diagnostics kernels");
     double v[k3DiagN];
     TRY3(cudaMemcpyAsync(v, c->dout, sizeof v, cudaMemcpyDeviceToHost, c->stream), "diagnostics read-back");
     TRY3(cudaStreamSynchronize(c->stream), "diagnostics");
