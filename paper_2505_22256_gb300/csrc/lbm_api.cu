@@ -438,7 +438,7 @@ void free_ctx(Ctx& c) {
         if (c.xout[k]) cudaFree(c.xout[k]);
     }
     void* ptrs[] = {c.dcases, c.f[0], c.f[1], c.flags, c.wsub, c.wa, c.solid, c.wl_node, c.wl_subst, c.wl_seff,
-                    c.wl_a, c.items, c.dense, c.fields, c.diag_part, c.diag_out, c.ca_work, c.ca_all, c.ca_batch, c.ca_points, c.fields_all, c.slide_list, c.tmaps, c.err, c.sched, c.gflags};
+                    c.wl_a, c.items, c.dense, c.fields, c.diag_part, c.diag_out, c.ca_work, c.ca_all, c.ca_batch, c.ca_points, c.fields_all, c.tmaps, c.err, c.sched, c.gflags};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (c.own_stream && c.stream) cudaStreamDestroy(c.stream);
@@ -584,20 +584,7 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
         if (p) cudaFree(p);
     if (st != LBM_OK) return bail(st);
 
-    // cases whose walls slide get the sliding-wall fix-up after every step
-    {
-        std::vector<int> sl;
-        for (int i = 0; i < ncases; ++i)
-            if (c.hcases[i].pf.moving) {
-                sl.push_back(i);
-                c.slide_max_nx = std::max(c.slide_max_nx, c.hcases[i].nx);
-            }
-        c.slide_n = (int)sl.size();
-        if (c.slide_n) {
-            STEP(dalloc(c, &c.slide_list, sl.size()), "sliding-wall list");
-            STEP(cudaMemcpy(c.slide_list, sl.data(), sl.size() * sizeof(int), cudaMemcpyHostToDevice), "sliding-wall list");
-        }
-    }
+    for (const DevCase& d : c.hcases) c.sliding = c.sliding || d.pf.moving;
 
     // work list and launch shape.  Block width: the one that launches fewer thread columns over all
     // cases (windows of width - 8 interior columns; 64 wins on lattices narrower than about 56
