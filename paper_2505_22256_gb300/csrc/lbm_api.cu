@@ -285,10 +285,11 @@ lbm_status build_items(Ctx& c) {
     const int W = c.block_threads, Wi = W - 8;
     lbm_status ts = build_tmaps(c);
     if (ts != LBM_OK) return ts;
-    int per_sm = 0;
-    CUDA_TRY(step_occupancy(c.storage, W, &per_sm));
-    if (per_sm < 1) return fail(LBM_ECUDA, "step kernel cannot be resident with %d threads", W);
+    int per_sm = 0, fields_per_sm = 0;
+    CUDA_TRY(step_occupancy(c.storage, W, &per_sm, &fields_per_sm));
+    if (per_sm < 1 || fields_per_sm < 1) return fail(LBM_ECUDA, "step kernel cannot be resident with %d threads", W);
     const long long resident = (long long)per_sm * c.num_sms;
+    c.fields_blocks = fields_per_sm * c.num_sms;
     const int ncases = (int)c.hcases.size();
     std::vector<int> nstrip(ncases);
     long long strips = 0;
@@ -588,7 +589,9 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
 
     // work list and launch shape.  Block width: the one that launches fewer thread columns over all
     // cases (windows of width - 8 interior columns; 64 wins on lattices narrower than about 56
-    // columns).  The wall-list correction is inlined where wall-list nodes are common (more than 4 %
+    // columns).  In 16-bit storage a column of the 64-wide form costs more, two-warp blocks hiding less
+    // of each other's latency: with about the same number of columns, 64 uneven cases ran at 149.3 us in it
+    // and at 134.9 in the 128-wide form.  The wall-list correction is inlined where wall-list nodes are common (more than 4 %
     // of the fluid nodes) or the lattices are large: the call's register saves cost every row
     // (seven 1024 x 1024 cases, 0.5 % wall-list nodes: 183 us called, 173 inlined; FP16 170 and 150;
     // 14 of 300 x 350 60.0 and 54.8).  Below about 2^18 nodes a step is a chain of latencies and the two
@@ -599,7 +602,8 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
         for (int w = 0; w < 2; ++w)
             for (const DevCase& d : c.hcases)
                 cols[w] += (long long)((d.nx + widths[w] - 9) / (widths[w] - 8)) * widths[w] * d.ny;
-        c.block_threads = cols[1] < cols[0] ? 64 : 128;
+        const double per_col = c.elem == 2 ? 1.08 : 1.0;
+        c.block_threads = per_col * cols[1] < cols[0] ? 64 : 128;
     }
     c.block_rows = 0;
     {

@@ -73,7 +73,8 @@ struct Ctx {
     int wall_inline = 0;             // step kernel variant: wall-list correction inline (1) or called (0)
     bool sliding = false;            // some case has sliding walls: the step kernel form that reflects them
     int rows_used = 0;
-    int grid_blocks = 0;
+    int grid_blocks = 0;             // blocks of the step launch, all resident
+    int fields_blocks = 0;           // resident blocks of the fields pass
     int4* items = nullptr;
     int nitems = 0;                  // step list: items [0, nitems)
     int nitems_all = 0;              // per-case lists follow: items [nitems, nitems_all)
@@ -133,7 +134,7 @@ cudaError_t launch_set_rest_all(Ctx& c, const double* rhoA_all, const double* rh
 cudaError_t launch_set_rest(Ctx& c, int case_index, const double* rhoA, const double* rhoB);
 cudaError_t launch_get_state(Ctx& c, int case_index, double* dense_f);
 int step_smem_bytes(int storage, int threads);
-cudaError_t step_occupancy(int storage, int threads, int* blocks_per_sm);
+cudaError_t step_occupancy(int storage, int threads, int* step_blocks, int* fields_blocks);
 int ghost_cols(int storage);      // ghost columns on each side of a stored population row
 int box_extra_cols(int storage);  // tensor-box columns beyond the block width
 

@@ -30,6 +30,8 @@
 // grid-wide synchronisation.
 #include <math.h>
 
+#include <type_traits>
+
 #include "lbm_internal.h"
 #include "lbm_tma.cuh"
 
@@ -103,6 +105,66 @@ __device__ __forceinline__ V2<R> load_v2(const Pair<S>* p, const Params<R>& P, i
 // and with global memory (state read-back).  The plain form assumes no blocked link and no open
 // column.  Pin: the rarely used constants (inlet).
 // ------------------------------------------------------------------------------------------------
+template <bool kAddShift, class S, class R>
+__device__ __forceinline__ void complete_open(bool inlet, bool outlet, const Params<R>& Pin, int y, V2<R> (&f)[9]) {
+    if (inlet) {  // non-equilibrium bounce-back about f^eq(rho_in, (u_in(y), 0))
+        R sc = (R)1;
+        if (Pin.inlet_profile) {  // Poiseuille profile of peak u_in (Sec. 3.3)
+            const R s = (R)y + (R)0.5;
+            sc = Pin.prof_c * s * ((R)Pin.ny - s);
+        }
+        const V2<R> s2 = vbc<R>(sc), d1 = V2<R>{Pin.d1[0], Pin.d1[1]}, d5 = V2<R>{Pin.d5[0], Pin.d5[1]};
+        f[1] = vfma(d1, s2, f[3]);
+        f[5] = vfma(d5, s2, f[7]);
+        f[8] = vfma(d5, s2, f[6]);
+    }
+    if (outlet && Pin.outlet) {
+        // Zou-He density condition per component (Sec. 3.3 outflow, pressure reading), replacing the
+        // f3, f6, f7 the copy rule pulled above: the node gets the densities rho_out and no momentum
+        // along y, with non-equilibrium bounce-back along x.  The known populations give
+        // rho u_x = f0 + f2 + f4 + 2 (f1 + f5 + f8) - rho_out; shifted storage holds h = f - w rho0,
+        // whose known sum misses rho0 (those weights sum to 1).
+        V2<R> known = vadd(vadd(vadd(f[0], f[2]), f[4]), vmul(vbc<R>(2), vadd(vadd(f[1], f[5]), f[8])));
+        if constexpr (Store<S>::kShift && !kAddShift) known = vadd(known, V2<R>{Pin.rho0[0], Pin.rho0[1]});
+        const V2<R> rho_ux = vsub(known, V2<R>{Pin.rho_out[0], Pin.rho_out[1]});
+        const V2<R> dy = vsub(f[2], f[4]);
+        const V2<R> c6 = vmul(vbc<R>(1.0 / 6.0), rho_ux);
+        f[3] = vsub(f[1], vmul(vbc<R>(2.0 / 3.0), rho_ux));
+        f[7] = vsub(vfma(vbc<R>(0.5), dy, f[5]), c6);
+        f[6] = vsub(vsub(f[8], vmul(vbc<R>(0.5), dy)), c6);
+    }
+}
+
+// The pairs of the pull as stored (16-bit storage): as pull(), before complete_open().
+template <bool kGeneral, class S>
+__device__ __forceinline__ void pull_stored(const Pair<S>* __restrict__ rm, const Pair<S>* __restrict__ r0,
+                                            const Pair<S>* __restrict__ rp, int ps, int c, uint16_t fl, bool inlet,
+                                            bool outlet, uint32_t (&h)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const Pair<S>* src = cy(i) > 0 ? rm : (cy(i) < 0 ? rp : r0);
+        int off = i * ps + c - cx(i);
+        if (kGeneral && i > 0) {
+            const bool blocked = (fl >> (i - 1)) & 1u;
+            int b = c;
+            if (cx(i) < 0 && outlet) b = (fl & kOutletOwnBit) ? c : c - 1;  // copied from upstream
+            // through the inlet: complete_open() replaces it; any pair of the row will do
+            const bool own = blocked || (cx(i) > 0 && inlet);
+            src = own ? r0 : src;
+            off = own ? opp(i) * ps + b : i * ps + b - cx(i);
+        }
+        h[i] = *reinterpret_cast<const uint32_t*>(src + off);
+    }
+}
+template <class S, class R>
+__device__ __forceinline__ void widen_stored(const uint32_t (&h)[9], V2<R> (&f)[9]) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const Pair<S> p = *reinterpret_cast<const Pair<S>*>(&h[i]);
+        load_pair<S, R>(&p, (R)0, (R)0, f[i].x, f[i].y);
+    }
+}
+
 template <bool kGeneral, class S, class R, class I, bool kAddShift = true>
 __device__ __forceinline__ void pull(const Pair<S>* __restrict__ rm, const Pair<S>* __restrict__ r0,
                                      const Pair<S>* __restrict__ rp, I ps, int c, uint16_t fl, bool inlet, bool outlet,
@@ -128,32 +190,7 @@ __device__ __forceinline__ void pull(const Pair<S>* __restrict__ rm, const Pair<
         }
         f[i] = load_v2<kAddShift, S, R>(src + off, P, i);
     }
-    if (kGeneral && inlet) {  // non-equilibrium bounce-back about f^eq(rho_in, (u_in(y), 0))
-        R sc = (R)1;
-        if (Pin.inlet_profile) {  // Poiseuille profile of peak u_in (Sec. 3.3)
-            const R s = (R)y + (R)0.5;
-            sc = Pin.prof_c * s * ((R)Pin.ny - s);
-        }
-        const V2<R> s2 = vbc<R>(sc), d1 = V2<R>{Pin.d1[0], Pin.d1[1]}, d5 = V2<R>{Pin.d5[0], Pin.d5[1]};
-        f[1] = vfma(d1, s2, f[3]);
-        f[5] = vfma(d5, s2, f[7]);
-        f[8] = vfma(d5, s2, f[6]);
-    }
-    if (kGeneral && outlet && Pin.outlet) {
-        // Zou-He density condition per component (Sec. 3.3 outflow, pressure reading), replacing the
-        // f3, f6, f7 the copy rule pulled above: the node gets the densities rho_out and no momentum
-        // along y, with non-equilibrium bounce-back along x.  The known populations give
-        // rho u_x = f0 + f2 + f4 + 2 (f1 + f5 + f8) - rho_out; shifted storage holds h = f - w rho0,
-        // whose known sum misses rho0 (those weights sum to 1).
-        V2<R> known = vadd(vadd(vadd(f[0], f[2]), f[4]), vmul(vbc<R>(2), vadd(vadd(f[1], f[5]), f[8])));
-        if constexpr (Store<S>::kShift && !kAddShift) known = vadd(known, V2<R>{Pin.rho0[0], Pin.rho0[1]});
-        const V2<R> rho_ux = vsub(known, V2<R>{Pin.rho_out[0], Pin.rho_out[1]});
-        const V2<R> dy = vsub(f[2], f[4]);
-        const V2<R> c6 = vmul(vbc<R>(1.0 / 6.0), rho_ux);
-        f[3] = vsub(f[1], vmul(vbc<R>(2.0 / 3.0), rho_ux));
-        f[7] = vsub(vfma(vbc<R>(0.5), dy, f[5]), c6);
-        f[6] = vsub(vsub(f[8], vmul(vbc<R>(0.5), dy)), c6);
-    }
+    if (kGeneral) complete_open<kAddShift, S, R>(inlet, outlet, Pin, y, f);
 }
 
 // Window column -> lattice column; -1 when it lies outside a wall boundary.
@@ -201,9 +238,12 @@ struct Diag {
     }
 };
 
-template <class R>
+// What a thread keeps of a row between its density pass and its collision two rows later: the nine
+// pulled pairs (f_i^A, f_i^B), in 16-bit storage as stored (nine registers, not 18; they are widened
+// again at the collision).
+template <class S, class R>
 struct RowState {
-    V2<R> f[9];  // (f_i^A, f_i^B)
+    typename std::conditional<sizeof(S) == 2, uint32_t, V2<R>>::type f[9];
     uint16_t fl;
     uint32_t sub;
     R ax, ay;
@@ -466,22 +506,25 @@ struct StepArgs {
     double *o_rA, *o_rB, *o_ux, *o_uy, *diag_part;
 };
 
-// blocks per SM the launch bounds ask for: the same registers per thread at either width.  16-bit
-// storage fits four 128-thread blocks per SM in shared memory (FP32 three, FP64 two), and needs the
-// warps: its launch is bound by instruction latency, not by DRAM.
+// blocks per SM the launch bounds ask for: the same registers per thread at either width.  FP32 and FP64
+// are held by shared memory and registers (three and two 128-thread blocks).  16-bit storage is bound by
+// instruction latency, not by DRAM, and needs the warps: with the pulled pairs kept as stored it fits 96
+// registers without a spill, five blocks (four blocks, values kept and the loop unrolled -> now, us per
+// step: 4096 x 2048 porous 281 -> 211, 2048 x 512 throat 37.9 -> 32.4, 64 uneven cases 153.6 -> 134.9,
+// seven 1024 x 1024 149.0 -> 149.7; four blocks of the new form 224, 33.4, -, 154; six spill: 477, 44.6, -, 348).
 #ifndef LBM_MIN_BLOCKS_16
-#define LBM_MIN_BLOCKS_16 4
+#define LBM_MIN_BLOCKS_16 5
 #endif
-template <class S, int T>
-constexpr int step_min_blocks() {
-    return (sizeof(S) == 8 ? 2 : sizeof(S) == 2 ? LBM_MIN_BLOCKS_16 : LBM_MIN_BLOCKS) * (128 / T);
-}
-
 // kStep: collide.  kFields: write the fields and their diagnostics instead.  kSlide: collide, with
 // sliding walls in some case (apart, since the few wall rows' code costs every row registers).
 enum { kStep = 0, kFieldsPass = 1, kSlide = 2 };
+// The fields pass holds more at once: four blocks in 16-bit storage, where five spill.
+template <class S, int kMode, int T>
+constexpr int step_min_blocks() {
+    return (sizeof(S) == 8 ? 2 : sizeof(S) == 4 ? LBM_MIN_BLOCKS : kMode == kFieldsPass ? 4 : LBM_MIN_BLOCKS_16) * (128 / T);
+}
 template <class S, class R, int kMode, bool kWallInline, int T>
-__global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a) {
+__global__ void __launch_bounds__(T, step_min_blocks<S, kMode, T>()) k_step(StepArgs a) {
     constexpr bool kFields = kMode == kFieldsPass;
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int kSlots = slots_of<S>();
@@ -584,7 +627,7 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
         };
 
         // densities of row r into the ring, populations of row r into st
-        auto rho_row = [&](int r, int m, RowState<R>& st) -> bool {
+        auto rho_row = [&](int r, int m, RowState<S, R>& st) -> bool {
             const bool ok = wait_next();  // f* row r+dir; rows r and r-dir sit in the two slots before
             const unsigned char* s0 = smem + so_0;
             // node flags of row r; rows beyond a wall boundary are solid
@@ -597,11 +640,20 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
                 const Pair<S>* rm = reinterpret_cast<const Pair<S>*>(smem + (dir > 0 ? so_m : so_p));
                 const Pair<S>* r0 = reinterpret_cast<const Pair<S>*>(s0);
                 const Pair<S>* rp = reinterpret_cast<const Pair<S>*>(smem + (dir > 0 ? so_p : so_m));
-                if (general) pull<true, S, R, int, false>(rm, r0, rp, BX, sc, st.fl, inlet, outlet, P, s_par, r, st.f);
-                else pull<false, S, R, int, false>(rm, r0, rp, BX, sc, st.fl, inlet, outlet, P, s_par, r, st.f);
+                V2<R> f[9];
+                if constexpr (sizeof(S) == 2) {
+                    if (general) pull_stored<true, S>(rm, r0, rp, BX, sc, st.fl, inlet, outlet, st.f);
+                    else pull_stored<false, S>(rm, r0, rp, BX, sc, st.fl, inlet, outlet, st.f);
+                    widen_stored<S, R>(st.f, f);
+                    if (inlet || outlet) complete_open<false, S, R>(inlet, outlet, s_par, r, f);
+                } else {
+                    if (general) pull<true, S, R, int, false>(rm, r0, rp, BX, sc, st.fl, inlet, outlet, P, s_par, r, st.f);
+                    else pull<false, S, R, int, false>(rm, r0, rp, BX, sc, st.fl, inlet, outlet, P, s_par, r, st.f);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) f[i] = st.f[i];
+                }
                 // rho_k = sum_i f_i as a balanced tree (short dependency chains); 16-bit storage sums
                 // h_i = f_i - w_i rho0 and adds rho0 once (the weights sum to 1)
-                const V2<R>* f = st.f;
                 rho2 = vadd(vadd(vadd(f[0], f[1]), vadd(f[2], f[3])),
                             vadd(vadd(f[4], f[5]), vadd(f[6], vadd(f[7], f[8]))));
                 if constexpr (Store<S>::kShift) rho2 = vadd(rho2, V2<R>{s_par.rho0[0], s_par.rho0[1]});
@@ -624,7 +676,7 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
 
         // collide row y (state st, complete gradient g[0]) and store it
         // lo: ring slot of row y - 2 (rows y-2 .. y+2 sit at slots lo .. lo+4)
-        auto update_row = [&](int y, int lo, const RowState<R>& st, const Grad<R>& g, Diag<R>& dg) {
+        auto update_row = [&](int y, int lo, const RowState<S, R>& st, const Grad<R>& g, Diag<R>& dg) {
             if (!interior || (st.fl & kSolidBit)) {
                 if constexpr (kFields) {
                     const long long o = (a.fields_global ? C.d_off : 0) + (long long)y * P.nx + x;
@@ -681,7 +733,20 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
             FAy += rA * P.gy;
             FBx += rB * P.gx;
             FBy += rB * P.gy;
-            const V2<R>* f = st.f;
+            V2<R> f[9];
+            if constexpr (sizeof(S) == 2) {
+                uint32_t h[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {  // opaque, or the compiler keeps the first widened values instead
+                    h[i] = st.f[i];
+                    asm volatile("" : "+r"(h[i]));
+                }
+                widen_stored<S, R>(h, f);
+                if (inlet || outlet) complete_open<false, S, R>(inlet, outlet, s_par, y, f);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) f[i] = st.f[i];
+            }
             // momentum per component, then summed over the components (Eq. 4)
             const V2<R> d13 = vsub(f[1], f[3]), d24 = vsub(f[2], f[4]), d57 = vsub(f[5], f[7]), d68 = vsub(f[6], f[8]);
             const V2<R> mx2 = vadd(d13, vsub(d57, d68)), my2 = vadd(d24, vadd(d57, d68));
@@ -749,7 +814,7 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
         if constexpr (kFields) dg.init();
         Grad<R> g;
         g.zero();
-        RowState<R> s0, s1, s2;
+        RowState<S, R> s0, s1, s2;
         s0.sub = s1.sub = s2.sub = 0;
         s0.ax = s0.ay = s1.ax = s1.ay = s2.ax = s2.ay = (R)0;
 
@@ -763,7 +828,7 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
 
         // One row of the march: densities of row q into `cur`, barrier, refill of the slot that
         // held f* row q-dir, gradient row sums of row q, collision of row q-2 dir (`old`).
-        auto iter = [&](int q, RowState<R>& old, RowState<R>& cur) -> bool {
+        auto iter = [&](int q, RowState<S, R>& old, RowState<S, R>& cur) -> bool {
             const int mq = ring_slot(q);
             const bool mine = rho_row(q, mq, cur);
             if (__syncthreads_or(!mine)) return false;
@@ -778,9 +843,21 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, T>()) k_step(StepArgs a)
             return true;
         };
 
-        // row states rotate with period three: row q goes into cur, row q-2 dir is old
+        // row states rotate with period three: row q goes into cur, row q-2 dir is old.  In FP32 and FP64
+        // the loop is unrolled over the period; in 16-bit storage a state is 13 registers, and moving two
+        // of them per row costs less than three copies of the row's code (instruction fetch).
         int q = dir > 0 ? y0 - 2 : y1 + 1;
         int left = (y1 - y0) + 4;  // rows of densities to produce
+        if constexpr (sizeof(S) == 2) {
+#pragma unroll 1
+            while (ok && left > 0) {
+                ok = iter(q, s0, s2);
+                q += dir;
+                --left;
+                s0 = s1;
+                s1 = s2;
+            }
+        } else
         while (ok && left > 0) {
             ok = iter(q, s0, s2);
             q += dir;
@@ -1066,22 +1143,18 @@ int step_smem_bytes(int storage, int threads) {
     }
 }
 
-cudaError_t step_occupancy(int storage, int threads, int* blocks_per_sm) {
+cudaError_t step_occupancy(int storage, int threads, int* step_blocks, int* fields_blocks) {
     const int bytes = step_smem_bytes(storage, threads);
+    *step_blocks = *fields_blocks = 1 << 30;  // per SM; of the step's forms the most restrictive one's
     for (int v = 0; v < 4; ++v) {
-        cudaError_t e =
-            cudaFuncSetAttribute(step_kernel(storage, v, threads), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-    }
-    // the most restrictive of the variants sets the resident blocks
-    int m = 1 << 30;
-    for (int v = 0; v < 4; ++v) {
+        void* k = step_kernel(storage, v, threads);
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         int b = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, step_kernel(storage, v, threads), threads, bytes);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k, threads, bytes);
         if (e != cudaSuccess) return e;
+        int& m = v == 2 ? *fields_blocks : *step_blocks;
         m = b < m ? b : m;
     }
-    *blocks_per_sm = m;
     return cudaSuccess;
 }
 
@@ -1099,7 +1172,7 @@ cudaError_t launch_fields(Ctx& c, int ci, double* rhoA, double* rhoB, double* ux
     double* o4[4] = {rhoA ? rhoA : c.fields, rhoB ? rhoB : c.fields + N, ux ? ux : c.fields + 2 * N,
                      uy ? uy : c.fields + 3 * N};
     const int n = C.item_end - C.item_begin;
-    const int grid = n < c.grid_blocks ? n : c.grid_blocks;
+    const int grid = n < c.fields_blocks ? n : c.fields_blocks;
     (void)diag;
     StepArgs a = make_args(c, C.item_begin, C.item_end, o4, c.diag_part);
     return dispatch(c, a, c.stream, true, grid);
@@ -1113,7 +1186,7 @@ cudaError_t launch_diag_reduce(Ctx& c, int ci) {
 cudaError_t launch_fields_all(Ctx& c, double* rhoA_all, double* rhoB_all, double* ux_all, double* uy_all) {
     double* o4[4] = {rhoA_all, rhoB_all, ux_all, uy_all};
     const int n = c.nitems_all - c.nitems;
-    const int grid = n < c.grid_blocks ? n : c.grid_blocks;
+    const int grid = n < c.fields_blocks ? n : c.fields_blocks;
     StepArgs a = make_args(c, c.nitems, c.nitems_all, o4, nullptr);
     a.fields_global = 1;
     return dispatch(c, a, c.stream, true, grid);
@@ -1126,7 +1199,7 @@ cudaError_t launch_densities_all(Ctx& c, double* rhoA_all, double* rhoB_all) {
 cudaError_t launch_diag_all(Ctx& c, double* rhoA_all, double* rhoB_all) {
     double* o4[4] = {rhoA_all, rhoB_all, nullptr, nullptr};  // densities too when given (all cases)
     const int n = c.nitems_all - c.nitems;
-    const int grid = n < c.grid_blocks ? n : c.grid_blocks;
+    const int grid = n < c.fields_blocks ? n : c.fields_blocks;
     StepArgs a = make_args(c, c.nitems, c.nitems_all, o4, c.diag_part);
     a.fields_global = 1;
     cudaError_t e = dispatch(c, a, c.stream, true, grid);
