@@ -21,6 +21,7 @@
 #include <stdarg.h>
 
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "lbm_internal.h"
@@ -264,8 +265,8 @@ struct Diag3 {
 // The density pairs (rho_A, rho_B) of the planes z-2 .. z+2 over the block's columns and a halo of
 // two on each side (36 x 8 sites per plane) sit in a six-plane shared-memory ring; solid sites
 // hold -1, so nodes near the wall take the second-layer copy and the solid switch out of the ring
-// as well.  Each thread loads its share of the halo of plane z+4 into registers one plane before
-// it enters the ring, and the flags of the next plane.  Per plane: pull of the node's 38
+// as well.  Each thread loads its share of the halo of plane z+3 into registers while plane z is
+// worked on, and the flags of the next plane.  Per plane: pull of the node's 38
 // populations, stencil sums out of the ring, moments, forces, collision, store; one barrier.  Both
 // components share each instruction: densities, gradients, forces and populations are (A, B) pairs.
 // ------------------------------------------------------------------------------------------------
@@ -337,6 +338,17 @@ __device__ __forceinline__ void wall_stencil3(const V2<R>* b0, const V2<R>* b1, 
 #ifndef LBM3_MIN_BLOCKS
 #define LBM3_MIN_BLOCKS 3
 #endif
+// Blocks per SM.  16-bit storage, whose DRAM time is half, waits for its pulls' latency: with the pulled
+// pairs held as stored behind the stencil sums (19 registers, not 38) and one density plane in flight it
+// fits 128 registers without a spill, four blocks (100 x 100 x 140: 120.0 -> 105.2 us a step, three blocks
+// of the same form 113.6; 200 x 200 x 280: 730 -> 637, 677).  FP32 spills at four and is slower (851 -> 897).
+#ifndef LBM3_MIN_BLOCKS_16
+#define LBM3_MIN_BLOCKS_16 4
+#endif
+template <class S>
+__host__ __device__ constexpr int march_blocks() {
+    return sizeof(S) == 8 ? 2 : (sizeof(S) == 2 ? LBM3_MIN_BLOCKS_16 : LBM3_MIN_BLOCKS);
+}
 // kMode: kStep collides.  The fields forms write rho_A, rho_B and u (FP64, each of o5 may be NULL) in
 // place of the collision; kFieldsDiag also adds each node's values to the thread's diagnostic record,
 // and each block writes one record (block index blockIdx.x + gridDim.x (blockIdx.y + gridDim.y
@@ -347,7 +359,7 @@ struct Out5 {
     double* p[5];
 };
 template <class S, class R, int kAdh, int kMode = kStep>
-__global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
+__global__ void __launch_bounds__(k3T, march_blocks<S>())
     k3_march(Geo3 g, P3<R> P, int zc, const uint32_t* __restrict__ flags, const Pair<S>* __restrict__ fs,
              const V2<R>* __restrict__ rho, Pair<S>* __restrict__ fout, Out5 o5, double* __restrict__ part) {
     using V = V2<R>;
@@ -386,7 +398,9 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
     const int yx = active ? y * g.nx + x : 0;
     const Nb3 nb(g, active ? x : 0, active ? y : 0, 0);
     // the node's 38 populations at plane z: f_i(x) = f*_i(x - e_i), or f*_opp(i)(x) across a blocked link
-    auto pull_plane = [&](int z, uint32_t fl, V (&f)[19]) {
+    // (16-bit storage: as stored; widened where they are used, behind the stencil sums)
+    using Held = typename std::conditional<sizeof(S) == 2, Pair<S>, V>::type;
+    auto pull_plane = [&](int z, uint32_t fl, Held (&f)[19]) {
         const int s = z * nxy + yx;
         const int zoff[3] = {wrapc(z - 1, g.nz) * nxy, z * nxy, wrapc(z + 1, g.nz) * nxy};
 #pragma unroll
@@ -399,7 +413,8 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
                 src = i == 0 ? s : zoff[1 - e3z(i)] + nb.yo[2 - e3y(i)] + nb.xw[2 - e3x(i)];
                 q = i;
             }
-            f[i] = ld3<S, R>(fs + (long long)q * g.N + src, P, q);
+            if constexpr (sizeof(S) == 2) f[i] = fs[(long long)q * g.N + src];
+            else f[i] = ld3<S, R>(fs + (long long)q * g.N + src, P, q);
         }
     };
 
@@ -416,19 +431,17 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
 #pragma unroll
         for (int d = 0; d < 5; ++d) store_plane(z0 - 2 + d, v[d]);
     }
-    V nxt[k3HN];
-    load_plane(z0 + 3, nxt);
     __syncthreads();
 
     for (int z = z0; z < z1; ++z) {
-        V nn[k3HN];
-        if (z + 4 <= z1 + 1) load_plane(z + 4, nn);  // planes up to z1 + 1 are needed
+        V nxt[k3HN];  // enters the ring when this plane is done; planes up to z1 + 1 are needed
+        if (z + 3 <= z1 + 1) load_plane(z + 3, nxt);
         const uint32_t fl = fl_nx;  // the flags are loaded one plane ahead
         if (z + 1 < z1 && active) fl_nx = flags[(z + 1) * nxy + yx];
         const int s = z * nxy + yx;
         if (!(fl & k3Solid)) {
-            V f[19];
-            pull_plane(z, fl, f);
+            Held held[19];
+            pull_plane(z, fl, held);
             // the node's stencil out of the ring: bs[d] = plane z - 2 + d at the node's column
             const V* bs[5];
 #pragma unroll
@@ -475,6 +488,12 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
                 } else {
                     GA = P.lam * P.Gw2;
                 }
+            }
+            V f[19];
+#pragma unroll
+            for (int i = 0; i < 19; ++i) {
+                if constexpr (sizeof(S) == 2) f[i] = ld3<S, R>(&held[i], P, i);  // opposite directions share w rho0
+                else f[i] = held[i];
             }
             // momentum per component from the differences of opposite populations (i odd, opp = i + 1)
             V mv[3] = {vbc<R>(0), vbc<R>(0), vbc<R>(0)};
@@ -553,8 +572,6 @@ __global__ void __launch_bounds__(k3T, sizeof(R) == 8 ? 2 : LBM3_MIN_BLOCKS)
         }
         if (z + 3 <= z1 + 1) store_plane(z + 3, nxt);
         __syncthreads();
-#pragma unroll
-        for (int k = 0; k < k3HN; ++k) nxt[k] = nn[k];
     }
     if constexpr (kDiag) {  // the block's record: warps by shuffles, then the warps in order
         __shared__ double red[k3T / 32][k3DiagN];
@@ -1355,7 +1372,8 @@ extern "C" lbm_status lbm3d_create(const lbm3d_grid* grid, const uint8_t* solid,
     }
     const dim3 gr = grid3(c->g);
     c->nparts = (long long)gr.x * gr.y * gr.z;
-    c->zc = zchunk3(c->g, (storage == LBM_STORE_F64 ? 2 : LBM3_MIN_BLOCKS) * prop.multiProcessorCount);
+    c->zc = zchunk3(c->g, (storage == LBM_STORE_F64 ? 2 : storage == LBM_STORE_F32 ? march_blocks<float>() : march_blocks<__half>()) *
+                               prop.multiProcessorCount);
     STEP3(cudaMalloc(&c->solid, N), "mask");
     STEP3(cudaMalloc(&c->flags, N * sizeof(uint32_t)), "flags");
     STEP3(cudaMalloc(&c->f[0], 38 * N * c->elem), "population buffer");
