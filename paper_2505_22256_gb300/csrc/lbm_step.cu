@@ -567,6 +567,10 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, kMode, T>()) k_step(Step
         for (int w = t; w < (int)(sizeof(Params<R>) / sizeof(int)); w += T) reinterpret_cast<int*>(&s_par)[w] = src[w];
     };
     int it = a.item_begin + (int)blockIdx.x;
+    // a launch with a block for every item claims nothing and leaves the counters alone: two atomics and
+    // a fence less at the end of a short launch (350 x 150 channel 8.0 -> 6.6 us a step, 2048 x 512 FP16
+    // 32.5 -> 30.9)
+    const bool claims = (int)gridDim.x < a.item_end - a.item_begin;
     if (it < a.item_end) copy_params(it);
     // everything above reads only what no kernel writes; the state, the counters and the outputs may
     // still be in use by the launch before this one
@@ -903,13 +907,14 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, kMode, T>()) k_step(Step
             }
             __syncthreads();
         }
+        if (!claims) break;
         if (t == 0) s_claim = a.item_begin + (int)gridDim.x + atomicAdd(a.sched, 1);
         __syncthreads();  // every thread is past the previous item's parameters, too
         it = s_claim;
         if (it < a.item_end) copy_params(it);
         __syncthreads();
     }
-    if (t == 0) {
+    if (claims && t == 0) {
         // the last block to finish sees every claim made and resets the counters for the next launch
         __threadfence();
         if (atomicAdd(a.sched + 1, 1) == (int)gridDim.x - 1) {
