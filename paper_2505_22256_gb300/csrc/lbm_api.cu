@@ -585,7 +585,8 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
         if (p) cudaFree(p);
     if (st != LBM_OK) return bail(st);
 
-    for (const DevCase& d : c.hcases) c.sliding = c.sliding || d.pf.moving;
+    for (const DevCase& d : c.hcases)
+        c.rare_form = c.rare_form || d.pf.moving || (d.bc_x == kPeriodic && d.nx < 2 * ghost_cols(storage));
 
     // work list and launch shape.  Block width: the one that launches fewer thread columns over all
     // cases (windows of width - 8 interior columns; 64 wins on lattices narrower than about 56

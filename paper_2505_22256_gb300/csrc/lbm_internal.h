@@ -71,7 +71,7 @@ struct Ctx {
     int block_threads = 128;
     int block_rows = 0;              // 0: automatic
     int wall_inline = 0;             // step kernel variant: wall-list correction inline (1) or called (0)
-    bool sliding = false;            // some case has sliding walls: the step kernel form that reflects them
+    bool rare_form = false;          // some case slides its walls or is periodic and under 2 ghost widths wide
     int rows_used = 0;
     int grid_blocks = 0;             // blocks of the step launch, all resident
     int fields_blocks = 0;           // resident blocks of the fields pass

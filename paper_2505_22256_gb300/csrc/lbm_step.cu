@@ -515,9 +515,11 @@ struct StepArgs {
 #ifndef LBM_MIN_BLOCKS_16
 #define LBM_MIN_BLOCKS_16 5
 #endif
-// kStep: collide.  kFields: write the fields and their diagnostics instead.  kSlide: collide, with
-// sliding walls in some case (apart, since the few wall rows' code costs every row registers).
-enum { kStep = 0, kFieldsPass = 1, kSlide = 2 };
+// kStep: collide.  kFieldsPass: write the fields and their diagnostics instead.  kRare: collide, in a
+// context where some case has sliding walls or is periodic and narrower than the ghost columns of both
+// sides (apart, since code for a few nodes costs every row registers: the second ghost copy alone 0.4 %
+// of the seven 1024 x 1024 cases).
+enum { kStep = 0, kFieldsPass = 1, kRare = 2 };
 // The fields pass holds more at once: four blocks in 16-bit storage, where five spill.
 template <class S, int kMode, int T>
 constexpr int step_min_blocks() {
@@ -790,7 +792,7 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, kMode, T>()) k_step(Step
                 collide<R, Store<S>::kShift>(f, r2, ux, uy, V2<R>{FAx, FBx}, V2<R>{FAy, FBy},
                                              V2<R>{P.omega[0], P.omega[1]}, V2<R>{P.cF[0], P.cF[1]}, o,
                                              V2<R>{s_par.om_rho0[0], s_par.om_rho0[1]});
-                if constexpr (kMode == kSlide) {
+                if constexpr (kMode == kRare) {
                     if (s_par.moving && (y == 0 || y == P.ny - 1)) slide_wall<S, R>(s_par, y != 0, o);
                 }
                 Pair<S>* out = fo + (long long)y * P.row + x + G;
@@ -809,6 +811,16 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, kMode, T>()) k_step(Step
                     for (int i = 0; i < 9; ++i) {
                         store_pair<S, R>(gout, o[i].x, o[i].y);
                         gout += P.plane;
+                    }
+                    if constexpr (kMode == kRare) {
+                        if (x < G && x >= P.nx - G) {  // narrower than 2 G: beyond the other edge, too
+                            gout = fo + (long long)y * P.row + (x - P.nx + G);
+#pragma unroll
+                            for (int i = 0; i < 9; ++i) {
+                                store_pair<S, R>(gout, o[i].x, o[i].y);
+                                gout += P.plane;
+                            }
+                        }
                     }
                 }
             }
@@ -1057,7 +1069,7 @@ void* kernel_ptr(int variant) {
         case 0: return (void*)k_step<S, R, kStep, false, T>;
         case 1: return (void*)k_step<S, R, kStep, true, T>;
         case 2: return (void*)k_step<S, R, kFieldsPass, true, T>;
-        default: return (void*)k_step<S, R, kSlide, true, T>;
+        default: return (void*)k_step<S, R, kRare, true, T>;
     }
 }
 
@@ -1066,7 +1078,7 @@ void* kernel_ptr_w(int variant, int threads) {
     return threads == 64 ? kernel_ptr<S, 64>(variant) : kernel_ptr<S, 128>(variant);
 }
 
-// variant 0: step, wall path out of line; 1: step, wall path inline; 2: fields pass; 3: step with sliding walls
+// variant 0: step, wall path out of line; 1: step, wall path inline; 2: fields pass; 3: the rare form
 void* step_kernel(int storage, int variant, int threads) {
     switch (storage) {
         case LBM_STORE_F64: return kernel_ptr_w<double>(variant, threads);
@@ -1111,7 +1123,7 @@ cudaError_t launch_step_w(const Ctx& c, const StepArgs& a, cudaStream_t s, bool 
     using R = typename ComputeOf<S>::type;
     const PdlLaunch l(dim3((unsigned)grid), dim3(T), smem_for<S>(T), s);
     if (fields) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kFieldsPass, true, T>, a);
-    if (c.sliding) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kSlide, true, T>, a);
+    if (c.rare_form) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kRare, true, T>, a);
     if (c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kStep, true, T>, a);
     return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kStep, false, T>, a);
 }
