@@ -14,8 +14,8 @@
 //             x + sign(e) (Sec. 2.4) and the solid switch; body force; velocity with Guo's
 //             half-force shift (Eq. 5); SRT collision with Guo forcing (Eqs. 1, 2, 6, 7) written to
 //             the other buffer.  Blocks march along z with the stencil's density planes in shared
-//             memory.  Its fields form (kFields) writes rho and u in FP64 and per-block diagnostic
-//             records instead of colliding.
+//             memory.  Its fields forms write rho and u in FP64 instead of colliding, one of them
+//             per-block diagnostic records, too.
 // Periodic in x, y and z.
 #include <math.h>
 #include <stdarg.h>
@@ -800,7 +800,8 @@ __device__ __forceinline__ bool phi3_pos_r(double a, double b) { return phi3_pos
 // Crossing links of every node.  The links of a node are tested by the signs of rho^e alone, a thread's
 // four nodes and their neighbours in flight together; flags and coordinates (a usable pair of nodes, no
 // pair across the periodic seam) are looked at only where a sign changes.  As part of a pass over all
-// nodes that looked at the flags first, one node after the other, it took 387 us on 200 x 200 x 280.
+// nodes that looked at the flags first, one node after the other, it took 387 us on 200 x 200 x 280
+// (the whole angle 0.95 ms; now 0.24 ms after the density pass).
 template <class R>
 __global__ void __launch_bounds__(kC3Threads) k3_ca_cross(Ca3<R> c) {
     const unsigned nx = c.g.nx, ny = c.g.ny, n = (unsigned)c.g.N;  // N < 2^31

@@ -47,7 +47,8 @@ constexpr int kRing = 6;
 // Rows of f* resident or in flight in shared memory (>= 4), per storage type: three rows feed a
 // pull, the rest are loads in flight.  FP32 takes six (on the seven-case sweep 0.1743 ms per launch
 // against 0.1772 with five; seven slots leave room for the 64-column form only); the 16-bit types
-// five (six measured 0.1533 against 0.1513 ms, four the same as five).
+// five (at five blocks per SM four measure the same, six the same on the sweep and 149 against 141 us
+// on 64 uneven cases).
 #ifndef LBM_SLOTS
 #define LBM_SLOTS 6
 #endif
