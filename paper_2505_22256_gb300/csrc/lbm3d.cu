@@ -178,9 +178,14 @@ __device__ __forceinline__ void pull3(const Geo3& g, const Nb3& nb, const Pair<S
     }
 }
 
+// k3_rho and k3_march follow each other as programmatic dependent launches: a block may be resident while
+// the launch before it still writes what this one reads (the populations fs, the densities rho).  So
+// those are plain coherent loads behind pdl_wait(), through pointers that promise nothing about the
+// kernel's lifetime: no __ldg and no __restrict__, either of which makes them read-only loads that the
+// compiler may move across the wait and that need not see the writes.  The flags never change.
 template <class S, class R>
-__global__ void __launch_bounds__(128) k3_rho(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags,
-                                              const Pair<S>* __restrict__ fs, typename Rho2<R>::T* __restrict__ rho) {
+__global__ void __launch_bounds__(128) k3_rho(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags, const Pair<S>* fs,
+                                              typename Rho2<R>::T* rho) {
     const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 4 + threadIdx.y, z = blockIdx.z;
     pdl_wait();
     pdl_launch_next();
@@ -360,8 +365,8 @@ struct Out5 {
 };
 template <class S, class R, int kAdh, int kMode = kStep>
 __global__ void __launch_bounds__(k3T, march_blocks<S>())
-    k3_march(Geo3 g, P3<R> P, int zc, const uint32_t* __restrict__ flags, const Pair<S>* __restrict__ fs,
-             const V2<R>* __restrict__ rho, Pair<S>* __restrict__ fout, Out5 o5, double* __restrict__ part) {
+    k3_march(Geo3 g, P3<R> P, int zc, const uint32_t* __restrict__ flags, const Pair<S>* fs, const V2<R>* rho,
+             Pair<S>* fout, Out5 o5, double* part) {
     using V = V2<R>;
     constexpr bool kFields = kMode != kStep, kDiag = kMode == kFieldsDiag;
     extern __shared__ __align__(16) unsigned char smem3[];
@@ -386,7 +391,7 @@ __global__ void __launch_bounds__(k3T, march_blocks<S>())
         const int zo = wrapc(p, g.nz) * nxy;
 #pragma unroll
         for (int k = 0; k < k3HN; ++k)
-            if (hoff[k] >= 0) v[k] = __ldg(rho + zo + hoff[k]);
+            if (hoff[k] >= 0) v[k] = rho[zo + hoff[k]];
     };
     auto slot = [&](int p) -> int { return wrapc(p % k3Ring, k3Ring); };  // ring slot of plane p >= -2
     auto store_plane = [&](int p, const V (&v)[k3HN]) {
