@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(kR3T) k3_set_rest(Geo3 g, P3<R> P, const uint3
             if (hoff[k] >= 0) ring[(z + 4) & 3][t + k * kR3T] = V{(R)(w19(7) * nA[k]), (R)(w19(7) * nB[k])};
     };
     const R lim = sizeof(R) == 8 ? (R)1e-290 : (R)1e-30;
-    auto tiny = [&](R q) { return q != (R)0 && q < lim && q > -lim; };
+    auto tiny = [&](R q) { return q < lim && q > -lim; };  // 0 too: twice what rounds to 0 need not
     load(z0 - 1);
     put(z0 - 1);
     load(z0);

@@ -255,10 +255,12 @@ __global__ void k_wall_scatter(const DevCase* __restrict__ cases, int c, const i
 // ------------------------------------------------------------------------------------------------
 constexpr int kRestT = 128, kRestW = kRestT - 2, kRestRows = 16;
 
-template <class R>
-__device__ __forceinline__ bool rest_tiny(R q) {  // nonzero and near the denormals of R
+// Near the denormals of R, or rounded to 0 (16 times what rounds to 0 need not).  With a storage shift
+// 0 is an ordinary value, rho = rho0, and a nonzero difference is far above the denormals.
+template <class S, class R>
+__device__ __forceinline__ bool rest_tiny(R q) {
     const R lim = sizeof(R) == 8 ? (R)1e-290 : (R)1e-30;
-    return q != (R)0 && q < lim && q > -lim;
+    return q < lim && q > -lim && !(Store<S>::kShift && q == (R)0);
 }
 
 template <class S>
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__
                 const V q = own ? ring[y & 3][t] : ring[(y + cy(i)) & 3][t + cx(i)];
                 const R up = (R)(i == 0 ? 16 : (i <= 4 ? 4 : 1));
                 V v{q.x * up, q.y * up};
-                if (rest_tiny(q.x) || rest_tiny(q.y)) {
+                if (!solid && (rest_tiny<S, R>(q.x) || rest_tiny<S, R>(q.y))) {
                     int tx = x, ty = y;
                     if (!own) {
                         tx += cx(i);
@@ -338,8 +340,12 @@ __global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__
                         ty += ty < 0 ? ny : (ty >= ny ? -ny : 0);
                     }
                     const long long z = (long long)ty * nx + tx;
-                    v = sol[z] ? V{(R)0, (R)0}
-                               : V{(R)(scaled(rA[z], 0) * (double)up), (R)(scaled(rB[z], 1) * (double)up)};
+                    double a = wq(i) * rA[z], b = wq(i) * rB[z];
+                    if constexpr (Store<S>::kShift) {
+                        a -= wq(i) * C.rho0[0];
+                        b -= wq(i) * C.rho0[1];
+                    }
+                    v = sol[z] ? V{(R)0, (R)0} : V{(R)a, (R)b};
                 }
                 if (solid) v = V{(R)0, (R)0};
                 store_pair<S, R>(o + i * plane, v.x, v.y);
