@@ -271,10 +271,16 @@ def kernel_source_hash(sources=KERNEL_SOURCES) -> str:
 STORE_TYPE = {"f32": "float, float", "f16": "__half, float", "bf16": "__nv_bfloat16, float", "f64": "double, double"}
 
 
-def step_kernel_name(storage: str, info: dict) -> str:
-    """The step kernel's template instantiation as ncu names it (storage type, compute type, fields
-    pass off, wall-list correction inlined or called, block width)."""
-    return f"k_step<{STORE_TYPE[storage]}, 0, {info['wall_inline']}, {info['block_threads']}>"
+def rare_form(cases) -> bool:
+    """Whether the context of these cases steps in the kernel's rare form: some case slides its walls, or
+    is periodic in x and narrower than the ghost columns of both sides (eight)."""
+    return any(tuple(c.u_wall) != (0.0, 0.0) or (c.bc_x == "periodic" and c.nx < 8) for c in cases)
+
+
+def step_kernel_name(storage: str, info: dict, rare: bool = False) -> str:
+    """The step kernel's template instantiation as ncu names it (storage type, compute type, form (0 step,
+    2 the rare form), wall-list correction inlined or called, block width)."""
+    return f"k_step<{STORE_TYPE[storage]}, {2 if rare else 0}, {info['wall_inline']}, {info['block_threads']}>"
 
 
 def counter_records(path: str) -> list[dict]:
@@ -484,7 +490,7 @@ def run_reference(args):
 LAUNCH_SHAPES = [(w, t, r) for w in (0, 1) for t in (128, 64) for r in (0, -8, -16, 16, 32, 64, 128)]
 
 
-def launch_table(args, lat, stream) -> int:
+def launch_table(args, cases, lat, stream) -> int:
     """Every launch shape the autotuner tries: one untimed and three single-launch steps each (under
     ncu, launch k of the capture belongs to shape k // 4 of the printed order), then, in a second
     pass, the mean time per launch over 16 steps in each shape.  Prints one JSON line."""
@@ -503,7 +509,7 @@ def launch_table(args, lat, stream) -> int:
         for _ in range(4):
             lat.step(1)
         shapes.append((w, t, r))
-        rows.append({"wall_inline": w, "block_threads": t, "rows_arg": r, "kernel": step_kernel_name(args.storage, info),
+        rows.append({"wall_inline": w, "block_threads": t, "rows_arg": r, "kernel": step_kernel_name(args.storage, info, rare_form(cases)),
                      "block_rows": info["block_rows"], "grid_blocks": info["grid_blocks"],
                      "work_items": info["work_items"]})
     for (w, t, r), row in zip(shapes, rows):
@@ -547,7 +553,7 @@ def storage_mode_line(args, cases, storage: str, stream) -> dict:
     algo = BYTES_PER_NODE[storage] * info["fluid_nodes"]
     peak, peak_kind = hbm_peak()
     traffic = committed_traffic(storage, info["nodes"], launch={
-        "workload": args.workload, "kernel": step_kernel_name(storage, info), "block_rows": info["block_rows"],
+        "workload": args.workload, "kernel": step_kernel_name(storage, info, rare_form(cases)), "block_rows": info["block_rows"],
         "grid_blocks": info["grid_blocks"]})
     return {"storage": storage, "value": info["nodes"] * MODE_STEPS * args.inner / (ms / 1e3) / 1e6, "unit": UNIT,
             "launch_ms": launch_ms, "steps_timed": MODE_STEPS * args.inner,
@@ -595,7 +601,7 @@ def run_ours(args):
     stream = torch.cuda.Stream()
     lat = lbm.Lattice(cases, storage=args.storage, cuda_stream=stream.cuda_stream)
     if args.launch_table:
-        return launch_table(args, lat, stream)
+        return launch_table(args, cases, lat, stream)
     # launch shape (row-chunk height, wall-list path) picked by the library's autotuner on the live
     # state, before the timed region
     tuned_ms = None if args.no_autotune else lbm.lbm_autotune(lat.ctx, 4)
@@ -655,7 +661,7 @@ def run_ours(args):
     achieved = algo_bytes / (launch_ms / 1e3) / 1e9
     peak, peak_kind = hbm_peak()
     traffic = committed_traffic(args.storage, nodes, launch={
-        "workload": args.workload, "kernel": step_kernel_name(args.storage, info), "block_rows": info["block_rows"],
+        "workload": args.workload, "kernel": step_kernel_name(args.storage, info, rare_form(cases)), "block_rows": info["block_rows"],
         "grid_blocks": info["grid_blocks"]})
     dall = lat.diagnostics_all(allow_unstable=True)
     d = dall[0]

@@ -1070,7 +1070,8 @@ void* kernel_ptr(int variant) {
         case 0: return (void*)k_step<S, R, kStep, false, T>;
         case 1: return (void*)k_step<S, R, kStep, true, T>;
         case 2: return (void*)k_step<S, R, kFieldsPass, true, T>;
-        default: return (void*)k_step<S, R, kRare, true, T>;
+        case 3: return (void*)k_step<S, R, kRare, true, T>;
+        default: return (void*)k_step<S, R, kRare, false, T>;
     }
 }
 
@@ -1079,7 +1080,9 @@ void* kernel_ptr_w(int variant, int threads) {
     return threads == 64 ? kernel_ptr<S, 64>(variant) : kernel_ptr<S, 128>(variant);
 }
 
-// variant 0: step, wall path out of line; 1: step, wall path inline; 2: fields pass; 3: the rare form
+// variant 0: step, wall path out of line; 1: step, wall path inline; 2: fields pass; 3, 4: the rare form
+// of the step with the wall path inline and out of line
+constexpr int kStepVariants = 5;
 void* step_kernel(int storage, int variant, int threads) {
     switch (storage) {
         case LBM_STORE_F64: return kernel_ptr_w<double>(variant, threads);
@@ -1124,7 +1127,8 @@ cudaError_t launch_step_w(const Ctx& c, const StepArgs& a, cudaStream_t s, bool 
     using R = typename ComputeOf<S>::type;
     const PdlLaunch l(dim3((unsigned)grid), dim3(T), smem_for<S>(T), s);
     if (fields) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kFieldsPass, true, T>, a);
-    if (c.rare_form) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kRare, true, T>, a);
+    if (c.rare_form && c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kRare, true, T>, a);
+    if (c.rare_form) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kRare, false, T>, a);
     if (c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kStep, true, T>, a);
     return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kStep, false, T>, a);
 }
@@ -1164,7 +1168,7 @@ int step_smem_bytes(int storage, int threads) {
 cudaError_t step_occupancy(int storage, int threads, int* step_blocks, int* fields_blocks) {
     const int bytes = step_smem_bytes(storage, threads);
     *step_blocks = *fields_blocks = 1 << 30;  // per SM; of the step's forms the most restrictive one's
-    for (int v = 0; v < 4; ++v) {
+    for (int v = 0; v < kStepVariants; ++v) {
         void* k = step_kernel(storage, v, threads);
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         int b = 0;
