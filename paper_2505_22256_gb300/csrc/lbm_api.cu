@@ -305,9 +305,9 @@ lbm_status build_items(Ctx& c) {
         return n;
     };
     const bool in_l2 = 2.0 * c.pop_elems * c.elem < 110e6;  // both state buffers, 129 MB of L2
-    auto uniform_cost = [&](int h) -> double {  // < 0: not resident at once
+    auto uniform_cost = [&](int h, long long at_once) -> double {  // < 0: more items than run at once
         const long long n = uniform_items(h);
-        return n <= resident ? one_round_cost(model, (double)n * W / 128.0 / c.num_sms, h, in_l2) : -1.0;
+        return n <= at_once ? one_round_cost(model, (double)n * W / 128.0 / c.num_sms, h, in_l2) : -1.0;
     };
     // rows of short chunks (Hs) per strip of case i for a given long height hb
     auto tail_chunks = [&](int i, int hb, int Hs) -> int {
@@ -343,7 +343,7 @@ lbm_status build_items(Ctx& c) {
         if (c.block_rows == 0) {
             best *= model.full;
             for (int h = 1; h <= 64; ++h) {
-                const double cost = uniform_cost(h);
+                const double cost = uniform_cost(h, resident);
                 if (cost >= 0 && cost < best) {
                     best = cost;
                     H = h;
@@ -365,10 +365,12 @@ lbm_status build_items(Ctx& c) {
         }
     }
     c.nitems = (int)items.size();
-    int Hr = 0;  // all per-case lists resident at once: the height that costs least, if any is
+    // The per-case lists run on the fields pass's blocks (four per SM in 16-bit storage, where the step has
+    // five).  All of them resident at once: the height that costs least, if any is.
+    int Hr = 0;
     double best_r = -1.0;
     for (int h = 1; h <= 16; ++h) {
-        const double cost = uniform_cost(h);
+        const double cost = uniform_cost(h, c.fields_blocks);
         if (cost >= 0 && (best_r < 0 || cost < best_r)) {
             best_r = cost;
             Hr = h;
@@ -376,11 +378,11 @@ lbm_status build_items(Ctx& c) {
     }
     for (int i = 0; i < ncases; ++i) {
         DevCase& d = c.hcases[i];
-        // per-case chunk height: minimise (items + resident) x (h + 5) for this case alone
+        // per-case chunk height: minimise (items + resident blocks) x (h + 5) for this case alone
         long long bestc = -1;
         int Hf = Hr > 0 ? Hr : 16;
         for (int h = 16; h <= 128 && Hr == 0; ++h) {
-            const long long cost = ((long long)nstrip[i] * ((d.ny + h - 1) / h) + resident) * (h + 5);
+            const long long cost = ((long long)nstrip[i] * ((d.ny + h - 1) / h) + c.fields_blocks) * (h + 5);
             if (bestc < 0 || cost < bestc) {
                 bestc = cost;
                 Hf = h;
