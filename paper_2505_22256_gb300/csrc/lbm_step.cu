@@ -637,8 +637,9 @@ __global__ void __launch_bounds__(T, step_min_blocks<S, kMode, T>()) k_step(Step
         auto rho_row = [&](int r, int m, RowState<S, R>& st) -> bool {
             const bool ok = wait_next();  // f* row r+dir; rows r and r-dir sit in the two slots before
             const unsigned char* s0 = smem + so_0;
-            // node flags of row r; rows beyond a wall boundary are solid
-            st.fl = (rcol && (P.bc_y == kPeriodic || (r >= 0 && r < P.ny)))
+            // node flags of row r; rows and columns beyond a wall boundary are solid (the loaded flags are 0,
+            // fluid, beyond their ghost columns, where a walled x has no column to pull from)
+            st.fl = (X >= 0 && (P.bc_y == kPeriodic || (r >= 0 && r < P.ny)))
                         ? reinterpret_cast<const uint16_t*>(s0 + plan.pop_bytes)[t + 6]
                         : kSolidBit;
             V2<R> rho2 = vbc<R>(0);
