@@ -690,20 +690,23 @@ __global__ void k3_set(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags, cons
 // 1.61 ms on 200 x 200 x 280 in FP32, where its 168 B per node take 0.28 ms of HBM time; now 0.36 ms).
 // A q so small that scaling it up could differ from rounding the larger product takes the direct form.
 //
-// A block of 32 x 8 columns marches along kR3Z planes of z; q of the plane ahead, with a halo of one
-// node, goes into a ring of four shared-memory planes, one barrier per plane.
+// A block of 32 x 8 columns marches along `planes` planes of z; q of the plane ahead, with a halo of one
+// node, goes into a ring of four shared-memory planes, one barrier per plane.  At most kR3Z planes, and
+// fewer where those do not fill the GPU (us, 16 planes -> this rule, FP32 / FP64:
+// 24 x 24 x 34 31.1 -> 6.4 / 51.3 -> 6.4, 40 x 40 x 56 34.7 -> 12.6 / 56.6 -> 13.3, 64^3 33.4 -> 16.8 / 57.3 -> 20.9).
 constexpr int kR3X = 32, kR3Y = 8, kR3T = kR3X * kR3Y, kR3Z = 16;
 constexpr int kR3HX = kR3X + 2, kR3P = kR3HX * (kR3Y + 2), kR3N = (kR3P + kR3T - 1) / kR3T;
 
 template <class S, class R>
-__global__ void __launch_bounds__(kR3T) k3_set_rest(Geo3 g, P3<R> P, const uint32_t* __restrict__ flags,
+__global__ void __launch_bounds__(kR3T) k3_set_rest(Geo3 g, P3<R> P, int planes,
+                                                    const uint32_t* __restrict__ flags,
                                                     const double* __restrict__ rA, const double* __restrict__ rB,
                                                     Pair<S>* __restrict__ fs) {
     using V = V2<R>;
     __shared__ V ring[4][kR3P];
     const int tx = threadIdx.x, ty = threadIdx.y, t = ty * kR3X + tx;
     const int x0 = blockIdx.x * kR3X, y0 = blockIdx.y * kR3Y, x = x0 + tx, y = y0 + ty;
-    const int z0 = blockIdx.z * kR3Z, z1 = min(z0 + kR3Z, g.nz);
+    const int z0 = blockIdx.z * planes, z1 = min(z0 + planes, g.nz);
     const bool active = x < g.nx && y < g.ny;
     const long long nxy = (long long)g.nx * g.ny;
     int hoff[kR3N];  // in-plane offsets of this thread's halo sites
@@ -728,8 +731,10 @@ __global__ void __launch_bounds__(kR3T) k3_set_rest(Geo3 g, P3<R> P, const uint3
         for (int k = 0; k < kR3N; ++k)
             if (hoff[k] >= 0) ring[(z + 4) & 3][t + k * kR3T] = V{(R)(w19(7) * nA[k]), (R)(w19(7) * nB[k])};
     };
-    const R lim = sizeof(R) == 8 ? (R)1e-290 : (R)1e-30;
-    auto tiny = [&](R q) { return q < lim && q > -lim; };  // 0 too: twice what rounds to 0 need not
+    auto tiny = [&](R q) {  // 0 too: twice what rounds to 0 need not
+        if constexpr (sizeof(R) == 8) return (__double2hiint(q) & 0x7fffffff) < (60 << 20);  // below 2^-963
+        else return q < (R)1e-30 && q > (R)-1e-30;
+    };
     load(z0 - 1);
     put(z0 - 1);
     load(z0);
@@ -1064,6 +1069,7 @@ struct lbm3d_ctx {
     unsigned char* f[2] = {nullptr, nullptr};
     int cur = 0;
     unsigned char* rho = nullptr;  // [N] density pairs in the compute type
+    int num_sms = 0;
     int zc = 0;                    // z planes per block of the march
     double* part = nullptr;        // per-block diagnostic records
     long long nparts = 0;
@@ -1249,9 +1255,12 @@ cudaError_t set_state3(lbm3d_ctx* c, const double* f, int buf) {
 cudaError_t set_rest3(lbm3d_ctx* c, const double* a, const double* b) {
     return with_types3(c->storage, [&](auto* s_, auto* r_) {
         TYPES3(s_, r_);
+        const long long tiles = (long long)((c->g.nx + kR3X - 1) / kR3X) * ((c->g.ny + kR3Y - 1) / kR3Y);
+        int planes = kR3Z;  // three blocks on every SM, if there are planes enough (128^3: 77 us, eight planes 80)
+        while (planes > 1 && tiles * ((c->g.nz + planes - 1) / planes) < 3LL * c->num_sms) planes /= 2;
         const dim3 gr((unsigned)((c->g.nx + kR3X - 1) / kR3X), (unsigned)((c->g.ny + kR3Y - 1) / kR3Y),
-                      (unsigned)((c->g.nz + kR3Z - 1) / kR3Z));
-        k3_set_rest<S, R><<<gr, dim3(kR3X, kR3Y), 0, c->stream>>>(c->g, p3_of<R>(c), c->flags, a, b, state3<S>(c, c->cur));
+                      (unsigned)((c->g.nz + planes - 1) / planes));
+        k3_set_rest<S, R><<<gr, dim3(kR3X, kR3Y), 0, c->stream>>>(c->g, p3_of<R>(c), planes, c->flags, a, b, state3<S>(c, c->cur));
         return cudaGetLastError();
     });
 }
@@ -1378,8 +1387,9 @@ extern "C" lbm_status lbm3d_create(const lbm3d_grid* grid, const uint8_t* solid,
     }
     const dim3 gr = grid3(c->g);
     c->nparts = (long long)gr.x * gr.y * gr.z;
+    c->num_sms = prop.multiProcessorCount;
     c->zc = zchunk3(c->g, (storage == LBM_STORE_F64 ? 2 : storage == LBM_STORE_F32 ? march_blocks<float>() : march_blocks<__half>()) *
-                               prop.multiProcessorCount);
+                               c->num_sms);
     STEP3(cudaMalloc(&c->solid, N), "mask");
     STEP3(cudaMalloc(&c->flags, N * sizeof(uint32_t)), "flags");
     STEP3(cudaMalloc(&c->f[0], 38 * N * c->elem), "population buffer");

@@ -250,33 +250,39 @@ __global__ void k_wall_scatter(const DevCase* __restrict__ cases, int c, const i
 // take 95 us of HBM time; now 150 us, most of it its stores.)  A q so small that scaling it up
 // could differ from rounding the larger product takes the direct form.
 //
-// A block of kRestT columns (one halo column on each side) marches down kRestRows rows; q of the row
-// ahead goes into a ring of four shared-memory rows, one barrier per row.
+// A block of T columns (one halo column on each side) marches down `rows` rows; q of the row ahead goes
+// into a ring of four shared-memory rows, one barrier per row.  A row takes a block about 1 us whatever the
+// lattice, so 16 rows (at most: each block reads two halo rows more) serve only where they fill the GPU;
+// a smaller lattice takes fewer, down to one, and one narrower than 30 columns blocks of 32.
+// us, 16 rows of 128 columns -> this rule, FP32 / FP64: 40 x 300 24.8 -> 6.3 / 37.5 -> 6.4, 200 of 16 x 16
+// 22.7 -> 7.6 / 35.2 -> 8.8, 9 x 5000 20.8 -> 10.4 / 35.0 -> 10.6, three 256 x 256 24.9 -> 12.5 / 41.0 -> 14.5.
 // ------------------------------------------------------------------------------------------------
-constexpr int kRestT = 128, kRestW = kRestT - 2, kRestRows = 16;
+constexpr int kRestRows = 16;
 
 // Near the denormals of R, or rounded to 0 (16 times what rounds to 0 need not).  With a storage shift
-// 0 is an ordinary value, rho = rho0, and a nonzero difference is far above the denormals.
+// 0 is an ordinary value, rho = rho0, and a nonzero difference is far above the denormals.  FP64 looks at
+// the exponent: a comparison would cost its pipe as much as a product.
 template <class S, class R>
 __device__ __forceinline__ bool rest_tiny(R q) {
-    const R lim = sizeof(R) == 8 ? (R)1e-290 : (R)1e-30;
-    return q < lim && q > -lim && !(Store<S>::kShift && q == (R)0);
+    if constexpr (sizeof(R) == 8) return (__double2hiint(q) & 0x7fffffff) < (60 << 20);  // below 2^-963
+    else return q < (R)1e-30 && q > (R)-1e-30 && !(Store<S>::kShift && q == (R)0);
 }
 
-template <class S>
-__global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__ cases, int G, long long base,
-                                                     const uint8_t* __restrict__ solid_all,
-                                                     const uint16_t* __restrict__ flags_all,
-                                                     const double* __restrict__ rhoA_all,
-                                                     const double* __restrict__ rhoB_all, Pair<S>* __restrict__ out_all) {
+template <class S, int T>
+__global__ void __launch_bounds__(T) k_set_rest(const DevCase* __restrict__ cases, int G, int rows, long long base,
+                                                const uint8_t* __restrict__ solid_all,
+                                                const uint16_t* __restrict__ flags_all,
+                                                const double* __restrict__ rhoA_all,
+                                                const double* __restrict__ rhoB_all, Pair<S>* __restrict__ out_all) {
     using R = typename ComputeOf<S>::type;
     using V = V2<R>;
-    __shared__ V ring[4][kRestT];
+    constexpr int W = T - 2;
+    __shared__ V ring[4][T];
     const DevCase& C = cases[blockIdx.y];
     const int nx = C.nx, ny = C.ny, bcx = C.bc_x, t = threadIdx.x;
-    const int nstrip = (nx + kRestW - 1) / kRestW;
-    const int chunk = blockIdx.x / nstrip, xs = (blockIdx.x % nstrip) * kRestW;
-    const int y0 = chunk * kRestRows, y1 = min(y0 + kRestRows, ny);
+    const int nstrip = (nx + W - 1) / W;
+    const int chunk = blockIdx.x / nstrip, xs = (blockIdx.x % nstrip) * W;
+    const int y0 = chunk * rows, y1 = min(y0 + rows, ny);
     if (y0 >= ny) return;  // the grid covers the case with the most tiles
     const long long plane = C.pitch, row = 9 * plane;
     const double* rA = rhoA_all + (C.d_off - base);
@@ -288,7 +294,7 @@ __global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__
     const int x = xs - 1 + t;  // window column
     int X = x;                 // its lattice column, -1 outside a closed or open edge (never pulled from)
     if (x < 0 || x >= nx) X = bcx != kPeriodic ? -1 : (x < 0 ? x + nx : x % nx);
-    const bool mine = t >= 1 && t <= kRestW && x < nx;
+    const bool mine = t >= 1 && t <= W && x < nx;
 
     auto scaled = [&](double r, int k) -> double {
         double v = wq(5) * r;
@@ -303,10 +309,11 @@ __global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__
             r += r < 0 ? ny : -ny;
         }
         if (X < 0) return;
-        const long long s = (long long)r * nx + X;
-        if (sol[s]) return;
-        nA = rA[s];
-        nB = rB[s];
+        const long long s = (long long)r * nx + X;  // three loads in flight together
+        const bool is_solid = sol[s] != 0;
+        const double a = rA[s], b = rB[s];
+        nA = is_solid ? 0.0 : a;
+        nB = is_solid ? 0.0 : b;
     };
     auto put = [&](int r) { ring[r & 3][t] = V{(R)scaled(nA, 0), (R)scaled(nB, 1)}; };
     load(y0 - 1);
@@ -314,13 +321,16 @@ __global__ void __launch_bounds__(kRestT) k_set_rest(const DevCase* __restrict__
     load(y0);
     put(y0);
     load(y0 + 1);
+    uint16_t next_fl = mine ? flags[(long long)y0 * nx + x] : 0;
     for (int y = y0; y < y1; ++y) {
+        const uint16_t fl = next_fl;
         put(y + 1);
-        if (y + 1 < y1) load(y + 2);
+        if (y + 1 < y1) {
+            load(y + 2);
+            if (mine) next_fl = flags[(long long)(y + 1) * nx + x];
+        }
         __syncthreads();
         if (mine) {
-            const long long s = (long long)y * nx + x;
-            const uint16_t fl = flags[s];
             const bool solid = (fl & kSolidBit) != 0;
             Pair<S>* o = out + y * row + x + G;
             const bool gr = bcx == kPeriodic && x < G, gl = bcx == kPeriodic && x >= nx - G;  // ghost copies
@@ -396,24 +406,41 @@ cudaError_t launch_wall_cast(Ctx& c, int ci) {
     return cudaGetLastError();
 }
 
+template <class S>
+static void set_rest_launch(Ctx& c, dim3 g, int T, int rows, long long base, int c0, const double* rhoA, const double* rhoB) {
+    const int G = ghost_cols(c.storage);
+    Pair<S>* out = (Pair<S>*)c.f[c.cur];
+    if (T == 32) k_set_rest<S, 32><<<g, 32, 0, c.stream>>>(c.dcases + c0, G, rows, base, c.solid, c.flags, rhoA, rhoB, out);
+    else k_set_rest<S, 128><<<g, 128, 0, c.stream>>>(c.dcases + c0, G, rows, base, c.solid, c.flags, rhoA, rhoB, out);
+}
+
 // cases [c0, c0 + n) with the densities of case c at d_off - base
 static cudaError_t set_rest_cases(Ctx& c, int c0, int n, long long base, const double* rhoA, const double* rhoB) {
-    const int G = ghost_cols(c.storage);
+    int widest = 0;
+    for (int i = c0; i < c0 + n; ++i) widest = widest > c.hcases[i].nx ? widest : c.hcases[i].nx;
+    const int T = widest <= 30 ? 32 : 128;
+    auto tiles_of = [&](const DevCase& h, int rows) {
+        return (long long)((h.nx + T - 3) / (T - 2)) * ((h.ny + rows - 1) / rows);
+    };
+    int rows = kRestRows;  // 1,024 threads on every SM, if there are rows enough
+    for (; rows > 1; rows /= 2) {
+        long long all = 0;
+        for (int i = c0; i < c0 + n; ++i) all += tiles_of(c.hcases[i], rows);
+        if (all * T >= 1024LL * c.num_sms) break;
+    }
     for (const int end = c0 + n; c0 < end; c0 += 65535) {  // cases along gridDim.y, at most 65535 per launch
         const int m = end - c0 < 65535 ? end - c0 : 65535;
         long long tiles = 1;
         for (int i = c0; i < c0 + m; ++i) {
-            const DevCase& h = c.hcases[i];
-            const long long k = (long long)((h.nx + kRestW - 1) / kRestW) * ((h.ny + kRestRows - 1) / kRestRows);
+            const long long k = tiles_of(c.hcases[i], rows);
             tiles = tiles > k ? tiles : k;
         }
         const dim3 g((unsigned)tiles, (unsigned)m);
-        const DevCase* dc = c.dcases + c0;
         switch (c.storage) {
-            case LBM_STORE_F64: k_set_rest<double><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<double>*)c.f[c.cur]); break;
-            case LBM_STORE_F32: k_set_rest<float><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<float>*)c.f[c.cur]); break;
-            case LBM_STORE_F16_SHIFTED: k_set_rest<__half><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<__half>*)c.f[c.cur]); break;
-            default: k_set_rest<__nv_bfloat16><<<g, kRestT, 0, c.stream>>>(dc, G, base, c.solid, c.flags, rhoA, rhoB, (Pair<__nv_bfloat16>*)c.f[c.cur]); break;
+            case LBM_STORE_F64: set_rest_launch<double>(c, g, T, rows, base, c0, rhoA, rhoB); break;
+            case LBM_STORE_F32: set_rest_launch<float>(c, g, T, rows, base, c0, rhoA, rhoB); break;
+            case LBM_STORE_F16_SHIFTED: set_rest_launch<__half>(c, g, T, rows, base, c0, rhoA, rhoB); break;
+            default: set_rest_launch<__nv_bfloat16>(c, g, T, rows, base, c0, rhoA, rhoB); break;
         }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
