@@ -233,8 +233,8 @@ lbm_status build_tmaps(Ctx& c) {
     return LBM_OK;
 }
 
-// What a launch of the step kernel costs, in rows marched by a block that has its SM to itself (about
-// 0.9 us in FP32, 1.1 in 16-bit storage, 10.7 in FP64, where the FP64 pipe sets the pace).  An item
+// What a launch of the step kernel costs, in rows marched by a 128-column block that has its SM to itself
+// (about 0.9 us in FP32, 1.1 in 16-bit storage, 10.7 in FP64, where the FP64 pipe sets the pace).  An item
 // costs its rows plus `fill` (halo rows, first loads).  Blocks that share an SM slow each other by
 // `shared` while the state stays in L2 and by `spilled` when it does not; `full` scales the guided
 // list's estimate, which counts its last short item whole, to the same unit.  Fitted to uniform lists of 1- to 32-row items on fifteen lattices.
@@ -245,9 +245,15 @@ RowCost row_cost(int storage) {
     if (storage == LBM_STORE_F64) return {1.3, 2.0, 2.0, 1.8};
     return storage == LBM_STORE_F32 ? RowCost{4.5, 1.3, 1.6, 0.92} : RowCost{4.5, 1.5, 1.7, 0.92};
 }
-// n items of h rows that are all resident at once; blocks: items per SM, in blocks of 128 threads
-double one_round_cost(const RowCost& m, double blocks, int h, bool in_l2) {
-    return (h + m.fill) * (blocks <= 1.0 ? 1.0 : (in_l2 ? m.shared : m.spilled));
+// n items of h rows that are all resident at once, in blocks of `width` threads.  A 64-column block in FP64
+// neither takes half a 128-column one's time (alone 0.88 of it: its chain of FP64 latencies is as long) nor
+// slows its neighbours as much: up to three on an SM 1.15, four 1.55.  us a step, counted as half a
+// 128-column block -> so: 64 channels of 50 x 100 405 -> 254, 602 x 581 320 -> 232, 56 x 4000 235 -> 161.
+double one_round_cost(const RowCost& m, bool f64, int width, long long n, int sms, int h, bool in_l2) {
+    const double per_sm = (double)n / sms, blocks = per_sm * width / 128.0;
+    double slow = blocks <= 1.0 ? 1.0 : (in_l2 ? m.shared : m.spilled);
+    if (f64 && width == 64) slow = per_sm <= 1.0 ? 0.88 : (per_sm <= 3.0 ? 1.15 : 1.55);
+    return (h + m.fill) * slow;
 }
 
 // Row chunks [y0, y1) of one case's column strips, chunk-major; odd chunks march upwards (sign bit
@@ -307,7 +313,7 @@ lbm_status build_items(Ctx& c) {
     const bool in_l2 = 2.0 * c.pop_elems * c.elem < 110e6;  // both state buffers, 129 MB of L2
     auto uniform_cost = [&](int h, long long at_once) -> double {  // < 0: more items than run at once
         const long long n = uniform_items(h);
-        return n <= at_once ? one_round_cost(model, (double)n * W / 128.0 / c.num_sms, h, in_l2) : -1.0;
+        return n <= at_once ? one_round_cost(model, c.storage == LBM_STORE_F64, W, n, c.num_sms, h, in_l2) : -1.0;
     };
     // rows of short chunks (Hs) per strip of case i for a given long height hb
     auto tail_chunks = [&](int i, int hb, int Hs) -> int {
