@@ -356,7 +356,8 @@ lbm_status lbm_selftest_wait_timeout(lbm_ctx* ctx, double limit_ms);
 /* Choose the step kernel's form for wall-list nodes (the second-layer correction of Table 1): 1
  * inlines it (faster where wall-list nodes are common, e.g. porous media), 0 calls an out-of-line
  * copy.  lbm_create picks 1 when wall-list nodes exceed 4 % of the fluid nodes or the cases hold more
- * than 2^18 nodes; lbm_autotune tries both.  Results agree to FP rounding.
+ * than 2^18 nodes, 0 where cases with sliding walls or periodic ones under eight columns wide hold most
+ * of the nodes; lbm_autotune tries both.  Results agree to FP rounding.
  * Drops the captured graph.  LBM_EINVAL for other values. */
 lbm_status lbm_set_wall_path(lbm_ctx* ctx, int32_t inline_correction);
 

@@ -593,18 +593,22 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
         if (p) cudaFree(p);
     if (st != LBM_OK) return bail(st);
 
+    long long rare_nodes = 0;  // of the cases that need the rare form
     for (const DevCase& d : c.hcases)
-        c.rare_form = c.rare_form || d.pf.moving || (d.bc_x == kPeriodic && d.nx < 2 * ghost_cols(storage));
+        if (d.pf.moving || (d.bc_x == kPeriodic && d.nx < 2 * ghost_cols(storage))) rare_nodes += (long long)d.nx * d.ny;
+    c.rare_form = rare_nodes > 0;
 
     // work list and launch shape.  Block width: the one that launches fewer thread columns over all
     // cases (windows of width - 8 interior columns; 64 wins on lattices narrower than about 56
     // columns).  In 16-bit storage a column of the 64-wide form costs more, two-warp blocks hiding less
     // of each other's latency: with about the same number of columns, 64 uneven cases ran at 149.3 us in it
     // and at 134.9 in the 128-wide form.  The wall-list correction is inlined where wall-list nodes are common (more than 4 %
-    // of the fluid nodes) or the lattices are large: the call's register saves cost every row
-    // (seven 1024 x 1024 cases, 0.5 % wall-list nodes: 183 us called, 173 inlined; FP16 170 and 150;
-    // 14 of 300 x 350 60.0 and 54.8).  Below about 2^18 nodes a step is a chain of latencies and the two
-    // measure the same.
+    // of the fluid nodes) or the lattices are large: the call's register saves cost every row (us called,
+    // inlined: FP32 seven 1024 x 1024 183, 172.5; 14 of 300 x 350 54.8, 52.7; five 512 x 512 45.3, 44.9; 4096 x 2048
+    // porous 287, 255.  FP16 146.2, 147.2; 48.4, 47.0; 41.0, 38.2; 223, 211).  Below about 2^18 nodes a step
+    // is a chain of latencies and the two measure the same.  Sliding walls and narrow lattices have whole
+    // rows of wall-list nodes, which the call costs once per warp: where such cases hold most of the nodes it is
+    // called (FP32 64 channels of 160 x 200 64.8, 70.0; 512 of 50 x 100 98.0, 101.9; 6 x 100000 140, 151; FP16 the same).
     {
         long long cols[2] = {0, 0};
         const int widths[2] = {128, 64};
@@ -618,7 +622,8 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
     {
         long long fl = 0;
         for (const HostCase& h : c.cases) fl += h.nfluid;
-        c.wall_inline = ((double)c.nwall > 0.04 * (double)fl || c.dense_elems > (1LL << 18)) ? 1 : 0;
+        const bool mostly_rare = 2 * rare_nodes > c.dense_elems;
+        c.wall_inline = (!mostly_rare && ((double)c.nwall > 0.04 * (double)fl || c.dense_elems > (1LL << 18))) ? 1 : 0;
     }
     st = build_items(c);
     if (st != LBM_OK) return bail(st);
