@@ -281,6 +281,10 @@ void push_chunks(std::vector<int4>& out, int ci, int nstrip, int Wi, int y_begin
 //    With block_rows = 0 (the default), the cheapest by row_cost of that list with 8- and with
 //    16-row short chunks and of the uniform chunks that are all resident at once: a lattice that cannot
 //    fill the GPU in 16-row items is a serial chain of rows on a few SMs, and shorter items spread it.
+//    The 8-row tail has to promise 2 %: the estimate counts five halo rows per item and no more, and where it
+//    promises less the 16-row tail runs faster (us, tails of 8 / 16 rows: FP16 seven 1024 x 1024 150.1 / 147.2,
+//    64 uneven 135.5 / 134.8, porous 4096 x 2048 211.6 / 210.8, FP32 five 900 x 900 103.6 / 102.3; where it promises
+//    4 % and more: FP32 14 of 300 x 350 52.6 / 54.7, FP16 porous 2048 x 1020 70.9 / 73.5, 14 of 300 x 350 46.8 / 50.5).
 //    us per step, 16-row items -> this rule: 96 x 96 FP64 183 -> 28, FP32 19.9 -> 6.4, 350 x 150 open
 //    25.7 -> 8.0, 300 x 350 20.8 -> 10.2, four of them 26.5 -> 19.1, 512 x 512 21.5 -> 13.4, 14 of 300 x 350
 //    54.8 -> 52.7, 2048 x 512 FP16 38.0 -> 36.0.  The uniform chunks all march down, so a small case alone
@@ -338,7 +342,7 @@ lbm_status build_items(Ctx& c) {
                     tail += (double)nstrip[i] * ns * (short_h + 5.0);
                 }
                 const double cost = work / resident + (short_h + 5) + std::max(0.0, (hb + 5) - tail / resident);
-                if (best < 0 || cost < (short_h == Hs ? best : 0.997 * best)) {
+                if (best < 0 || cost < (short_h == Hs ? best : 0.98 * best)) {
                     best = cost;
                     Hb = hb;
                     Hs = short_h;
