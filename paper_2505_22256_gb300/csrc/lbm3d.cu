@@ -1193,8 +1193,8 @@ dim3 march_grid(const Geo3& g, int zc) {
 template <class S, class R>
 cudaError_t launch_rho3(lbm3d_ctx* c) {
     const PdlLaunch l(grid3(c->g), kBlock3, 0, c->stream);
-    return cudaLaunchKernelEx(&l.cfg, k3_rho<S, R>, c->g, p3_of<R>(c), (const uint32_t*)c->flags,
-                              (const Pair<S>*)state3<S>(c, c->cur), reinterpret_cast<typename Rho2<R>::T*>(c->rho));
+    return l.launch(k3_rho<S, R>, c->g, p3_of<R>(c), (const uint32_t*)c->flags, (const Pair<S>*)state3<S>(c, c->cur),
+                    reinterpret_cast<typename Rho2<R>::T*>(c->rho));
 }
 
 // the march over the whole lattice; the density pass comes first
@@ -1207,15 +1207,15 @@ cudaError_t launch_march3(lbm3d_ctx* c, const Out5& o5) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k3_march_smem<R>());
         if (e != cudaSuccess) return e;
     }
-    return cudaLaunchKernelEx(&l.cfg, kern, c->g, P, c->zc, (const uint32_t*)c->flags, (const Pair<S>*)state3<S>(c, c->cur),
-                              (const V2<R>*)c->rho, state3<S>(c, 1 - c->cur), o5, c->part);
+    return l.launch(kern, c->g, P, c->zc, (const uint32_t*)c->flags, (const Pair<S>*)state3<S>(c, c->cur),
+                    (const V2<R>*)c->rho, state3<S>(c, 1 - c->cur), o5, c->part);
 }
 
 template <class S, class R>
 cudaError_t step_once(lbm3d_ctx* c) {
     cudaError_t e = launch_rho3<S, R>(c);
     if (e == cudaSuccess) e = launch_march3<S, R, kStep>(c, Out5{});
-    c->cur ^= 1;
+    if (e == cudaSuccess) c->cur ^= 1;
     return e;
 }
 

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace lbm {
 
 // ------------------------------------------------------------------------------------------------
@@ -323,6 +325,13 @@ struct PdlLaunch {
         cfg.stream = s;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
+    }
+    // A refused launch is reported once, here: left behind, its error would be the next launch's.
+    template <class... P, class... A>
+    cudaError_t launch(void (*kernel)(P...), A&&... args) const {
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e;
     }
     PdlLaunch(const PdlLaunch&) = delete;
     PdlLaunch& operator=(const PdlLaunch&) = delete;

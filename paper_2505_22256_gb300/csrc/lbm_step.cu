@@ -1126,11 +1126,11 @@ template <class S, int T>
 cudaError_t launch_step_w(const Ctx& c, const StepArgs& a, cudaStream_t s, bool fields, int grid) {
     using R = typename ComputeOf<S>::type;
     const PdlLaunch l(dim3((unsigned)grid), dim3(T), smem_for<S>(T), s);
-    if (fields) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kFieldsPass, true, T>, a);
-    if (c.rare_form && c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kRare, true, T>, a);
-    if (c.rare_form) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kRare, false, T>, a);
-    if (c.wall_inline) return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kStep, true, T>, a);
-    return cudaLaunchKernelEx(&l.cfg, k_step<S, R, kStep, false, T>, a);
+    if (fields) return l.launch(k_step<S, R, kFieldsPass, true, T>, a);
+    if (c.rare_form && c.wall_inline) return l.launch(k_step<S, R, kRare, true, T>, a);
+    if (c.rare_form) return l.launch(k_step<S, R, kRare, false, T>, a);
+    if (c.wall_inline) return l.launch(k_step<S, R, kStep, true, T>, a);
+    return l.launch(k_step<S, R, kStep, false, T>, a);
 }
 
 template <class S>
