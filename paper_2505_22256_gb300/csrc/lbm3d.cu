@@ -345,7 +345,8 @@ __device__ __forceinline__ void wall_stencil3(const V2<R>* b0, const V2<R>* b1, 
 #endif
 // Blocks per SM.  16-bit storage, whose DRAM time is half, waits for its pulls' latency: with the pulled
 // pairs held as stored behind the stencil sums (19 registers, not 38) and one density plane in flight it
-// fits 128 registers without a spill, four blocks (100 x 100 x 140: 120.0 -> 105.2 us a step, three blocks
+// fits 128 registers, four blocks (no spill in the step but for 8 bytes with the D3Q19 adhesion; the fields
+// forms spill up to 136 bytes) (100 x 100 x 140: 120.0 -> 105.2 us a step, three blocks
 // of the same form 113.6; 200 x 200 x 280: 730 -> 637, 677).  FP32 spills at four and is slower (851 -> 897).
 #ifndef LBM3_MIN_BLOCKS_16
 #define LBM3_MIN_BLOCKS_16 4
@@ -1141,7 +1142,7 @@ const dim3 kBlock3(32, 4, 1);
 // z planes per block of the march.  A block costs its planes plus about 2 (the first density planes, the
 // start), and a launch runs its blocks in rounds of `resident`; about 16 planes, spread evenly over
 // nz, once there are many rounds (32 measured the same).  With 16 planes for every lattice a small
-// one ran as a few blocks: 40 x 40 x 56, 80 blocks, 39 us a step; with this rule 18.
+// one ran as a few blocks: 40 x 40 x 56, 80 blocks, 39 us a step; with this rule 17.
 #ifndef LBM3_ZCHUNK
 #define LBM3_ZCHUNK 16
 #endif

@@ -237,7 +237,8 @@ lbm_status build_tmaps(Ctx& c) {
 // (about 0.9 us in FP32, 1.1 in 16-bit storage, 10.7 in FP64, where the FP64 pipe sets the pace).  An item
 // costs its rows plus `fill` (halo rows, first loads).  Blocks that share an SM slow each other by
 // `shared` while the state stays in L2 and by `spilled` when it does not; `full` scales the guided
-// list's estimate, which counts its last short item whole, to the same unit.  Fitted to uniform lists of 1- to 32-row items on fifteen lattices.
+// list's estimate, which counts its last short item whole, to the same unit.  Fitted to uniform lists of 1- to 32-row items on fifteen lattices and
+// checked on 23, up to 64 rows (profiles/row_plan.md).
 struct RowCost {
     double fill, shared, spilled, full;
 };
@@ -283,11 +284,11 @@ void push_chunks(std::vector<int4>& out, int ci, int nstrip, int Wi, int y_begin
 //    fill the GPU in 16-row items is a serial chain of rows on a few SMs, and shorter items spread it.
 //    The 8-row tail has to promise 2 %: the estimate counts five halo rows per item and no more, and where it
 //    promises less the 16-row tail runs faster (us, tails of 8 / 16 rows: FP16 seven 1024 x 1024 150.1 / 147.2,
-//    64 uneven 135.5 / 134.8, porous 4096 x 2048 211.6 / 210.8, FP32 five 900 x 900 103.6 / 102.3; where it promises
-//    4 % and more: FP32 14 of 300 x 350 52.6 / 54.7, FP16 porous 2048 x 1020 70.9 / 73.5, 14 of 300 x 350 46.8 / 50.5).
-//    us per step, 16-row items -> this rule: 96 x 96 FP64 183 -> 28, FP32 19.9 -> 6.4, 350 x 150 open
-//    25.7 -> 8.0, 300 x 350 20.8 -> 10.2, four of them 26.5 -> 19.1, 512 x 512 21.5 -> 13.4, 14 of 300 x 350
-//    54.8 -> 52.7, 2048 x 512 FP16 38.0 -> 36.0.  The uniform chunks all march down, so a small case alone
+//    64 uneven 135.5 / 134.4, porous 4096 x 2048 211.7 / 211.2, FP32 five 900 x 900 103.5 / 102.4; where it promises
+//    4 % and more: FP32 14 of 300 x 350 52.5 / 54.4, FP16 porous 2048 x 1020 70.9 / 73.4, 14 of 300 x 350 46.8 / 50.4).
+//    us per step, 16-row tail -> this rule (both on the present kernel): 96 x 96 FP64 179 -> 21.8, FP32 18.2 ->
+//    5.0, 350 x 150 open 24.4 -> 6.6, 300 x 350 19.9 -> 8.7, four of them 24.6 -> 17.5, 512 x 512 20.5 -> 12.3,
+//    14 of 300 x 350 54.7 -> 52.7, 2048 x 512 FP16 35.6 -> 30.9.  The uniform chunks all march down, so a small case alone
 //    and the same case in a small ensemble reach the same bits at any height.
 //  * Per-case list (after the step list): uniform chunks, contiguous per case, used by the fields
 //    pass, whose per-item partial sums are reduced per case in item order.
@@ -314,7 +315,8 @@ lbm_status build_items(Ctx& c) {
         for (int i = 0; i < ncases; ++i) n += (long long)nstrip[i] * ((c.hcases[i].ny + h - 1) / h);
         return n;
     };
-    const bool in_l2 = 2.0 * c.pop_elems * c.elem < 110e6;  // both state buffers, 129 MB of L2
+    // both state buffers, beside what flags, wall data and stores in flight take (110 of GB300's 135.5 MB)
+    const bool in_l2 = 2.0 * c.pop_elems * c.elem < 0.81 * c.l2_bytes;
     auto uniform_cost = [&](int h, long long at_once) -> double {  // < 0: more items than run at once
         const long long n = uniform_items(h);
         return n <= at_once ? one_round_cost(model, c.storage == LBM_STORE_F64, W, n, c.num_sms, h, in_l2) : -1.0;
@@ -483,6 +485,7 @@ lbm_status create_impl(int ncases, const lbm_case* cs, int storage, void* stream
     c.elem = elem_size(storage);
     c.device = dev;
     c.num_sms = prop.multiProcessorCount;
+    c.l2_bytes = prop.l2CacheSize;
     auto bail = [&](lbm_status s) {
         free_ctx(c);
         delete h;

@@ -308,7 +308,7 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 // pdl_launch_next() lets the launch after this one start the same way; it comes after the wait, so
 // at most one launch waits behind the running one.  Per step this takes 1 to 3 us (the gap between
 // launches and the setup): 96 x 96 in one-row items 7.3 -> 6.3 us, 350 x 150 open channel 28.6 ->
-// 25.7 us, seven 1024 x 1024 cases 185 -> 182.5 us, with the sliding-wall pass 20.0 -> 18.9 us.
+// 25.7 us, seven 1024 x 1024 cases 185 -> 182.5 us.
 // ------------------------------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

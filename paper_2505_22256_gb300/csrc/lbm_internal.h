@@ -40,6 +40,7 @@ struct Ctx {
     bool own_stream = false;
     int device = 0;
     int num_sms = 0;
+    double l2_bytes = 0.0;
     long alloc_count = 0;            // allocations made through dalloc (failure-injection hook)
 
     std::vector<HostCase> cases;
