@@ -238,7 +238,7 @@ lbm_status build_tmaps(Ctx& c) {
 // costs its rows plus `fill` (halo rows, first loads).  Blocks that share an SM slow each other by
 // `shared` while the state stays in L2 and by `spilled` when it does not; `full` scales the guided
 // list's estimate, which counts its last short item whole, to the same unit.  Fitted to uniform lists of 1- to 32-row items on fifteen lattices and
-// checked on 23, up to 64 rows (profiles/row_plan.md).
+// checked on 23, up to 64 rows.
 struct RowCost {
     double fill, shared, spilled, full;
 };
